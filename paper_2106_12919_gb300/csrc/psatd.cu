@@ -469,9 +469,13 @@ __global__ void __launch_bounds__(256, sizeof(C) == 8 ? (VAR == 2 ? 2 : 4) : (VA
   }
   const uint32_t Nx = (uint32_t)u.coef.nx, Ny = (uint32_t)u.coef.ny;
   const int nmx = (qx == 0 || 2 * qx == Nx) ? 1 : 2, nmy = (qy == 0 || 2 * qy == Ny) ? 1 : 2;
-  for (int a = 0; a < nmx; ++a) {
+  // gridDim.y == 4: this thread takes the mirror (blockIdx.y >> 1, blockIdx.y & 1) only
+  const bool split = gridDim.y == 4;
+  const int a0 = split ? blockIdx.y >> 1 : 0, a1 = split ? min(nmx, a0 + 1) : nmx;
+  const int b0 = split ? blockIdx.y & 1 : 0, b1 = split ? min(nmy, b0 + 1) : nmy;
+  for (int a = a0; a < a1; ++a) {
     const uint32_t ix = a ? Nx - qx : qx;
-    for (int b = 0; b < nmy; ++b) {
+    for (int b = b0; b < b1; ++b) {
       const uint32_t iy = b ? Ny - qy : qy;
       const int64_t m = ((int64_t)ix * Ny + iy) * nzh + iz;
       update_one<VAR>(u, m, ix, iy, iz, cf);
@@ -877,10 +881,15 @@ pic_status psatd_update_t(pic_ctx* ctx, C* EB, C* J, const C* rn, const C* rp, C
   u.g_mode = g_mode;
   u.j_yee = j_yee;
   u.write_j = write_j;
-  const int bs = 256;
+  int bs = 256;
   const bool avg = ctx->variant == PIC_PSATD_AVERAGED_GALILEAN;
   if (ctx->coefq) {
-    const unsigned nb = (unsigned)((ctx->nq + bs - 1) / bs);
+    // One thread per table entry reads its coefficients once for up to four modes, but a small grid
+    // then has too few threads (32^3: 20 CTAs, 56 us in FP64, whose arithmetic runs at 1/64 rate): below
+    // two CTAs per SM a thread takes one mode, in CTAs of 64.
+    const bool split = ctx->nq < (int64_t)2 * 256 * ctx->nsm;
+    if (split) bs = 64;
+    const dim3 nb((unsigned)((ctx->nq + bs - 1) / bs), split ? 4 : 1);
     if (avg) update_quad_kernel<2, C, false><<<nb, bs, 0, ctx->stream>>>(u);
     else if (ctx->coefq_real) update_quad_kernel<0, C, true><<<nb, bs, 0, ctx->stream>>>(u);
     else update_quad_kernel<0, C, false><<<nb, bs, 0, ctx->stream>>>(u);
