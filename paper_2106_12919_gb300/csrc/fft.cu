@@ -27,18 +27,20 @@ namespace {
 
 constexpr int kZTile = 2048;             // complex elements per z-pass CTA (L lines * Nz/2)
 constexpr int kZThreads = kZTile / 8;    // one radix-8 butterfly per thread
+// the one-tile kernels' tile when 2048-element tiles would leave SMs idle (see z_small)
+constexpr int kZTileSmall = 512;
 
 using namespace pic_fft;
 
-// z-axis real-to-complex: L = 4096 / M lines of Nz = 2M reals -> M + 1 complex per line.  Each
+// z-axis real-to-complex: L = ZT / M lines of Nz = 2M reals -> M + 1 complex per line.  Each
 // thread loads its pass-0 butterfly (8 packed (even, odd) pairs, stride M / 8) straight from global
 // memory.
-template <class T, int LGM>
-__global__ void __launch_bounds__(kZThreads, (sizeof(T) == 4 ? 1536 : 1024) / kZThreads)
+template <class T, int LGM, int ZT>
+__global__ void __launch_bounds__(ZT / 8, (sizeof(T) == 4 ? 1536 : 1024) / (ZT / 8))
     fft_z_r2c_kernel(CRP6<T> in, CP6<typename Cplx<T>::type> out, int64_t nlines,
                      const typename Cplx<T>::type* __restrict__ tw, const typename Cplx<T>::type* __restrict__ twp) {
   using C = typename Cplx<T>::type;
-  constexpr int M = 1 << LGM, L = kZTile / M, lgnb = LGM - 3, nb = 1 << lgnb;
+  constexpr int M = 1 << LGM, L = ZT / M, lgnb = LGM - 3, nb = 1 << lgnb;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   const LayLine lay{zline_len(M)};
@@ -81,12 +83,12 @@ __global__ void __launch_bounds__(kZThreads, (sizeof(T) == 4 ? 1536 : 1024) / kZ
 
 // z-axis complex-to-real (unnormalised inverse); the imaginary parts of X_0, X_{Nz/2} are ignored.
 // The last pass writes its outputs straight to global memory.
-template <class T, int LGM>
-__global__ void __launch_bounds__(kZThreads, (sizeof(T) == 4 ? 1536 : 1024) / kZThreads)
+template <class T, int LGM, int ZT>
+__global__ void __launch_bounds__(ZT / 8, (sizeof(T) == 4 ? 1536 : 1024) / (ZT / 8))
     fft_z_c2r_kernel(CP6<typename Cplx<T>::type> in, RP6<T> out, int64_t nlines,
                      const typename Cplx<T>::type* __restrict__ tw, const typename Cplx<T>::type* __restrict__ twp) {
   using C = typename Cplx<T>::type;
-  constexpr int M = 1 << LGM, L = kZTile / M;
+  constexpr int M = 1 << LGM, L = ZT / M;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   const LayLine lay{zline_len(M)};
@@ -96,11 +98,11 @@ __global__ void __launch_bounds__(kZThreads, (sizeof(T) == 4 ? 1536 : 1024) / kZ
   constexpr int nzh = M + 1, P = M / 2 + 1, lgH = LGM - 1;
   // Z_k = (X_k + conj X_{M-k}) + i W^{-k} (X_k - conj X_{M-k})
   // k = 0 .. M/2 - 1 for every line (t < L M / 2), then k = M/2 (t >= L M / 2)
-  constexpr int kBatch = (L * P + kZThreads - 1) / kZThreads;
+  constexpr int kBatch = (L * P + (ZT / 8) - 1) / (ZT / 8);
   C xk[kBatch], xm[kBatch];
 #pragma unroll
   for (int q = 0; q < kBatch; ++q) {
-    const int t = threadIdx.x + q * kZThreads;
+    const int t = threadIdx.x + q * (ZT / 8);
     const bool mid = t >= (L << lgH);
     const int l = mid ? t - (L << lgH) : t >> lgH;
     const int k = mid ? (M >> 1) : t & ((M >> 1) - 1);
@@ -113,7 +115,7 @@ __global__ void __launch_bounds__(kZThreads, (sizeof(T) == 4 ? 1536 : 1024) / kZ
   }
 #pragma unroll
   for (int q = 0; q < kBatch; ++q) {
-    const int t = threadIdx.x + q * kZThreads;
+    const int t = threadIdx.x + q * (ZT / 8);
     if (t >= L * P) break;
     const bool mid = t >= (L << lgH);
     const int l = mid ? t - (L << lgH) : t >> lgH;
@@ -298,10 +300,16 @@ __global__ void __launch_bounds__(kZThreads, kZPipeCtasPerSm)
   }
 }
 
-// In-place C2C of length N = 2^LGN along a strided axis: element e of column col of outer line o
-// of component c at p[c] + o * os + e * es + col.  A CTA takes W = 2^LGW adjacent columns
-// (element-major tile, rows of W elements coalesced); pass 0 takes its inputs from global memory
-// and the last pass writes back to it.
+// In-place C2C of length N = 2^LGN along a strided axis.  The columns of a component are numbered
+// f = o * nc + col over the outer lines o and their nc columns, element e of column f at
+// p[c] + o * os + e * es + col.  A CTA takes W = 2^LGW consecutive column numbers (element-major tile,
+// rows of W elements coalesced, in two pieces where the group passes from one outer line to the
+// next); pass 0 takes its inputs from global memory and the last pass writes back to it.
+// Groups run over the outer lines because a half spectrum has Nz/2 + 1 columns: with groups of 16
+// kept inside one line the last of 2, 3, 5, 9, ... held a single column and cost as much as a full
+// one (the FP64 passes are bound by their arithmetic: 10 % of the pass at Nz = 256, 47 % at Nz = 32).
+// Measured: the FP64 field solve on 128x128x256 cells 9.47 -> 8.96 ms, one reverse step on 64^3 3.07 ->
+// 2.95 ms; FP32 runs 1 % or less (their idle columns moved no memory).
 // resident CTAs per SM the register cap is set for: ~1280 threads (FP32, 48 registers) or 1024 (FP64, 64)
 template <int T, int C_BYTES>
 struct StridedMinBlocks {
@@ -311,33 +319,35 @@ struct StridedMinBlocks {
 
 template <bool INV, class C, int LGN, int LGW>
 __global__ void __launch_bounds__((1 << (LGN + LGW)) / 8, (StridedMinBlocks<(1 << (LGN + LGW)) / 8, sizeof(C)>::value))
-    fft_strided_kernel(CP6<C> data, int64_t es, int64_t os, int ncols, const C* __restrict__ twp) {
+    fft_strided_kernel(CP6<C> data, int64_t es, int64_t os, uint32_t nc, uint32_t ncols, const C* __restrict__ twp) {
   constexpr int N = 1 << LGN, W = 1 << LGW, nb = N / 8;
   extern __shared__ __align__(16) unsigned char smraw[];
   C* sm = reinterpret_cast<C*>(smraw);
   const LayCol lay{LGW};
-  const int comp = blockIdx.z;
-  const int col0 = blockIdx.x * W;
-  C* base = data.p[comp] + (int64_t)blockIdx.y * os + col0;
-  const int wv = min(W, ncols - col0);
+  const int comp = blockIdx.y;
+  // every pass's butterflies of a thread lie in the column w of its thread index (LayCol::map)
   const int w = threadIdx.x & (W - 1), j = threadIdx.x >> LGW;
+  const uint32_t f = blockIdx.x * W + w;
+  const bool valid = f < ncols;
+  const uint32_t o = f / nc;
+  C* base = data.p[comp] + (int64_t)o * os + (f - o * nc);
   C v[8];
   {
-    const C* src = base + j * es + w;
+    const C* src = base + j * es;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = w < wv ? src[r * nb * es] : czero<C>();
+    for (int r = 0; r < 8; ++r) v[r] = valid ? src[r * nb * es] : czero<C>();
   }
   if constexpr (LGN == 3) {  // one radix-8 pass: registers to global memory
     dft<8, INV>(v);
-    if (w < wv) {
+    if (valid) {
 #pragma unroll
-      for (int r = 0; r < 8; ++r) base[r * es + w] = v[r];
+      for (int r = 0; r < 8; ++r) base[r * es] = v[r];
     }
   } else {
     pass0_from_regs<INV>(sm, lay, v, j, w);
     passes_ct<INV, LGN, 1, Plan<LGN>::npass - 1>(sm, lay, twp);
-    last_pass_to<INV, LGN>(sm, lay, twp, [&](int l, int e, C val) {
-      if (l < wv) base[e * es + l] = val;
+    last_pass_to<INV, LGN>(sm, lay, twp, [&](int, int e, C val) {
+      if (valid) base[e * es] = val;
     });
   }
 }
@@ -346,7 +356,7 @@ __global__ void __launch_bounds__((1 << (LGN + LGW)) / 8, (StridedMinBlocks<(1 <
 constexpr int strided_lgw(int lgN) { return lgN >= 10 ? 3 : 4; }
 
 template <class C>
-using StridedFn = void (*)(CP6<C>, int64_t, int64_t, int, const C*);
+using StridedFn = void (*)(CP6<C>, int64_t, int64_t, uint32_t, uint32_t, const C*);
 
 template <bool INV, class C, int LGN>
 StridedFn<C> strided_at() {
@@ -377,29 +387,29 @@ using ZC2RFn = void (*)(CP6<typename Cplx<T>::type>, RP6<T>, int64_t, const type
                         const typename Cplx<T>::type*);
 
 // the z kernels for M = Nz / 2 = 2^lgM (8 <= M <= 512)
-template <class T>
+template <class T, int ZT>
 ZR2CFn<T> z_r2c_fn(int lgM) {
   switch (lgM) {
-    case 3: return fft_z_r2c_kernel<T, 3>;
-    case 4: return fft_z_r2c_kernel<T, 4>;
-    case 5: return fft_z_r2c_kernel<T, 5>;
-    case 6: return fft_z_r2c_kernel<T, 6>;
-    case 7: return fft_z_r2c_kernel<T, 7>;
-    case 8: return fft_z_r2c_kernel<T, 8>;
-    case 9: return fft_z_r2c_kernel<T, 9>;
+    case 3: return fft_z_r2c_kernel<T, 3, ZT>;
+    case 4: return fft_z_r2c_kernel<T, 4, ZT>;
+    case 5: return fft_z_r2c_kernel<T, 5, ZT>;
+    case 6: return fft_z_r2c_kernel<T, 6, ZT>;
+    case 7: return fft_z_r2c_kernel<T, 7, ZT>;
+    case 8: return fft_z_r2c_kernel<T, 8, ZT>;
+    case 9: return fft_z_r2c_kernel<T, 9, ZT>;
   }
   return nullptr;
 }
-template <class T>
+template <class T, int ZT>
 ZC2RFn<T> z_c2r_fn(int lgM) {
   switch (lgM) {
-    case 3: return fft_z_c2r_kernel<T, 3>;
-    case 4: return fft_z_c2r_kernel<T, 4>;
-    case 5: return fft_z_c2r_kernel<T, 5>;
-    case 6: return fft_z_c2r_kernel<T, 6>;
-    case 7: return fft_z_c2r_kernel<T, 7>;
-    case 8: return fft_z_c2r_kernel<T, 8>;
-    case 9: return fft_z_c2r_kernel<T, 9>;
+    case 3: return fft_z_c2r_kernel<T, 3, ZT>;
+    case 4: return fft_z_c2r_kernel<T, 4, ZT>;
+    case 5: return fft_z_c2r_kernel<T, 5, ZT>;
+    case 6: return fft_z_c2r_kernel<T, 6, ZT>;
+    case 7: return fft_z_c2r_kernel<T, 7, ZT>;
+    case 8: return fft_z_c2r_kernel<T, 8, ZT>;
+    case 9: return fft_z_c2r_kernel<T, 9, ZT>;
   }
   return nullptr;
 }
@@ -454,6 +464,15 @@ bool z_pipe_ok(const pic_ctx* ctx, P const* p, int ncomp) {
   return true;
 }
 
+// Tiles of 2048 elements give a 32^3 grid 8 CTAs per component: 48 of 152 SMs with one CTA each, which
+// bounds the FP64 form (its arithmetic runs at 1/64 of the FP32 rate: 14.5 us per pass of 6
+// components).  Below two such tiles per SM the z passes run the one-tile kernels on 512-element tiles.
+// With the column groups of the strided passes and the split update: 10 FP64 steps on 32^3 3.32 ->
+// 2.74 ms, an 8-step gradient there 20.8 -> 19.1 ms.
+bool z_small(const pic_ctx* ctx, int ncomp) {
+  return (ctx->N[0] * ctx->N[1] * (ctx->N[2] / 2) / kZTile) * ncomp < 2 * ctx->nsm;
+}
+
 template <class C> const C* twiddles(const pic_ctx* ctx, int a);
 template <> const double2* twiddles<double2>(const pic_ctx* ctx, int a) { return ctx->twid[a]; }
 template <> const float2* twiddles<float2>(const pic_ctx* ctx, int a) { return ctx->twid32[a]; }
@@ -466,22 +485,16 @@ pic_status launch_strided(pic_ctx* ctx, CP6<C> d, int axis, bool inv, int ncomp)
   const int N = (int)ctx->N[axis];
   const int lgN = __builtin_ctz((unsigned)N);
   const int W = 1 << strided_lgw(lgN);
-  const int nzh = (int)ctx->nzh;
-  int64_t es, os, nouter;
-  if (axis == 1) {  // y: outer = x
-    es = nzh;
-    os = ctx->N[1] * nzh;
-    nouter = ctx->N[0];
-  } else {  // x: outer = y
-    es = ctx->N[1] * nzh;
-    os = nzh;
-    nouter = ctx->N[1];
-  }
+  // y: the outer lines are the x planes, of nzh columns each; x: one line of Ny * nzh columns
+  // (at most 2^30 columns, like the grid's cells)
+  const int64_t es = axis == 1 ? ctx->nzh : ctx->N[1] * ctx->nzh, os = ctx->N[1] * ctx->nzh;
+  const int64_t nc = axis == 1 ? ctx->nzh : ctx->N[1] * ctx->nzh;
+  const int64_t ncols = axis == 1 ? ctx->N[0] * ctx->nzh : nc;
   StridedFn<C> fn = inv ? strided_fn<true, C>(lgN) : strided_fn<false, C>(lgN);
   if (!fn) return pic_set_error(ctx, PIC_ERR_UNSUPPORTED, "transform length %d", N);
-  dim3 grid((nzh + W - 1) / W, (unsigned)nouter, ncomp);
+  dim3 grid((unsigned)((ncols + W - 1) / W), ncomp);
   const size_t smem = N > 8 ? (size_t)W * N * sizeof(C) : 0;
-  fn<<<grid, W * N / 8, smem, ctx->stream>>>(d, es, os, nzh, pass_twiddles<C>(ctx));
+  fn<<<grid, W * N / 8, smem, ctx->stream>>>(d, es, os, (uint32_t)nc, (uint32_t)ncols, pass_twiddles<C>(ctx));
   PIC_LAUNCH_CHECK(ctx);
   return PIC_OK;
 }
@@ -492,8 +505,8 @@ pic_status set_smem_attrs(pic_ctx* ctx) {
   using C = typename Cplx<T>::type;
   for (int lgM = 3; lgM <= 9; ++lgM) {
     const int zsm = (kZTile >> lgM) * zline_len(1 << lgM) * (int)sizeof(C);
-    PIC_CUDA_TRY(ctx, cudaFuncSetAttribute(z_r2c_fn<T>(lgM), cudaFuncAttributeMaxDynamicSharedMemorySize, zsm));
-    PIC_CUDA_TRY(ctx, cudaFuncSetAttribute(z_c2r_fn<T>(lgM), cudaFuncAttributeMaxDynamicSharedMemorySize, zsm));
+    PIC_CUDA_TRY(ctx, cudaFuncSetAttribute(z_r2c_fn<T, kZTile>(lgM), cudaFuncAttributeMaxDynamicSharedMemorySize, zsm));
+    PIC_CUDA_TRY(ctx, cudaFuncSetAttribute(z_c2r_fn<T, kZTile>(lgM), cudaFuncAttributeMaxDynamicSharedMemorySize, zsm));
   }
   if (sizeof(T) == 4) {
     for (int lgM = 3; lgM <= 9; ++lgM) {
@@ -587,12 +600,12 @@ template <class T>
 pic_status fft_r2c(pic_ctx* ctx, CRP6<T> in, CP6<typename Cplx<T>::type> out, int ncomp) {
   using C = typename Cplx<T>::type;
   const int Nz = (int)ctx->N[2];
-  const int L = z_lines_per_cta(Nz);
   const int64_t nlines = ctx->N[0] * ctx->N[1];
   const int lgM = __builtin_ctz((unsigned)(Nz / 2));
   if (lgM < 3 || lgM > 9) return pic_set_error(ctx, PIC_ERR_UNSUPPORTED, "transform length %d", Nz);
   if constexpr (sizeof(T) == 4) {
-    if (z_pipe_ok(ctx, in.p, ncomp)) {
+    if (!z_small(ctx, ncomp) && z_pipe_ok(ctx, in.p, ncomp)) {
+      const int L = z_lines_per_cta(Nz);
       const int tpc = (int)((nlines + L - 1) / L);
       const ZPipe zp{nlines, tpc, tpc * ncomp, ctx->dev_err};
       const int grid = std::min(zp.ntiles, kZPipeCtasPerSm * ctx->nsm);
@@ -605,10 +618,12 @@ pic_status fft_r2c(pic_ctx* ctx, CRP6<T> in, CP6<typename Cplx<T>::type> out, in
       return launch_strided<C>(ctx, out, 0, false, ncomp);
     }
   }
-  dim3 grid((unsigned)((nlines + L - 1) / L), ncomp);
-  const size_t smem = (size_t)L * zline_len(Nz / 2) * sizeof(C);
-  z_r2c_fn<T>(lgM)<<<grid, kZThreads, smem, ctx->stream>>>(in, out, nlines, twiddles<C>(ctx, 2),
-                                                            pass_twiddles<C>(ctx));
+  const bool small = z_small(ctx, ncomp);
+  const int zt = small ? kZTileSmall : kZTile, Lz = zt / (Nz / 2);
+  dim3 grid((unsigned)((nlines + Lz - 1) / Lz), ncomp);
+  const size_t smem = (size_t)Lz * zline_len(Nz / 2) * sizeof(C);
+  (small ? z_r2c_fn<T, kZTileSmall>(lgM) : z_r2c_fn<T, kZTile>(lgM))<<<grid, zt / 8, smem, ctx->stream>>>(
+      in, out, nlines, twiddles<C>(ctx, 2), pass_twiddles<C>(ctx));
   PIC_LAUNCH_CHECK(ctx);
   pic_status st = launch_strided<C>(ctx, out, 1, false, ncomp);
   if (st != PIC_OK) return st;
@@ -623,12 +638,12 @@ pic_status fft_c2r(pic_ctx* ctx, CP6<typename Cplx<T>::type> in, RP6<T> out, int
   st = launch_strided<C>(ctx, in, 1, true, ncomp);
   if (st != PIC_OK) return st;
   const int Nz = (int)ctx->N[2];
-  const int L = z_lines_per_cta(Nz);
   const int64_t nlines = ctx->N[0] * ctx->N[1];
   const int lgM = __builtin_ctz((unsigned)(Nz / 2));
   if (lgM < 3 || lgM > 9) return pic_set_error(ctx, PIC_ERR_UNSUPPORTED, "transform length %d", Nz);
   if constexpr (sizeof(T) == 4) {
-    if (z_pipe_ok(ctx, in.p, ncomp)) {
+    if (!z_small(ctx, ncomp) && z_pipe_ok(ctx, in.p, ncomp)) {
+      const int L = z_lines_per_cta(Nz);
       const int tpc = (int)((nlines + L - 1) / L);
       const ZPipe zp{nlines, tpc, tpc * ncomp, ctx->dev_err};
       const int grid = std::min(zp.ntiles, kZPipeCtasPerSm * ctx->nsm);
@@ -639,10 +654,12 @@ pic_status fft_c2r(pic_ctx* ctx, CP6<typename Cplx<T>::type> in, RP6<T> out, int
       return PIC_OK;
     }
   }
-  dim3 grid((unsigned)((nlines + L - 1) / L), ncomp);
-  const size_t smem = (size_t)L * zline_len(Nz / 2) * sizeof(C);
-  z_c2r_fn<T>(lgM)<<<grid, kZThreads, smem, ctx->stream>>>(in, out, nlines, twiddles<C>(ctx, 2),
-                                                            pass_twiddles<C>(ctx));
+  const bool small = z_small(ctx, ncomp);
+  const int zt = small ? kZTileSmall : kZTile, Lz = zt / (Nz / 2);
+  dim3 grid((unsigned)((nlines + Lz - 1) / Lz), ncomp);
+  const size_t smem = (size_t)Lz * zline_len(Nz / 2) * sizeof(C);
+  (small ? z_c2r_fn<T, kZTileSmall>(lgM) : z_c2r_fn<T, kZTile>(lgM))<<<grid, zt / 8, smem, ctx->stream>>>(
+      in, out, nlines, twiddles<C>(ctx, 2), pass_twiddles<C>(ctx));
   PIC_LAUNCH_CHECK(ctx);
   return PIC_OK;
 }
