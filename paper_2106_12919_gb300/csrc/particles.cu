@@ -79,8 +79,9 @@ __device__ __forceinline__ void push_u(const PushArgs& a, int64_t p, const doubl
     return;
   }
   const double umx = a.ux[p] + k * f[0], umy = a.uy[p] + k * f[1], umz = a.uz[p] + k * f[2];
-  const double gm = sqrt(1.0 + (umx * umx + umy * umy + umz * umz) * a.inv_c2);
-  const double tx = k * f[3] / gm, ty = k * f[4] / gm, tz = k * f[5] / gm;
+  // (one rsqrt instead of a square root and three divisions: FP64 divisions cost about ten operations)
+  const double igm = rsqrt(1.0 + (umx * umx + umy * umy + umz * umz) * a.inv_c2);
+  const double tx = k * f[3] * igm, ty = k * f[4] * igm, tz = k * f[5] * igm;
   const double s2 = 2.0 / (1.0 + tx * tx + ty * ty + tz * tz);
   const double sx = s2 * tx, sy = s2 * ty, sz = s2 * tz;
   const double upx = umx + (umy * tz - umz * ty);
@@ -91,9 +92,11 @@ __device__ __forceinline__ void push_u(const PushArgs& a, int64_t p, const doubl
   uz = umz + (upx * sy - upy * sx) + k * f[2];
 }
 
+// x in [0, L) after a move of less than a period; the comparisons are on the bit patterns (of positive
+// doubles, ordered as integers), off the FP64 pipe
 __device__ __forceinline__ double wrap(double x, double L) {
-  if (x >= L) x -= L;
-  if (x < 0.0) x += L;
+  if (__double_as_longlong(x) >= __double_as_longlong(L)) x -= L;  // x >= L > 0 (or not finite)
+  if (__double_as_longlong(x) < 0 && x < 0.0) x += L;
   return x;
 }
 
@@ -172,7 +175,7 @@ __device__ __forceinline__ void push_particle(const PushArgs& a, int64_t p) {
   // push u^{n-1/2} -> u^{n+1/2}
   double ux, uy, uz;
   push_u(a, p, f, ux, uy, uz);
-  const double ig = 1.0 / sqrt(1.0 + (ux * ux + uy * uy + uz * uz) * a.inv_c2);
+  const double ig = rsqrt(1.0 + (ux * ux + uy * uy + uz * uz) * a.inv_c2);
   const double vx = ux * ig, vy = uy * ig, vz = uz * ig;
   // move: x^{n+1} = x^n + dt (v - v_gal); J at x^{n+1/2}
   const double dX = a.dt * (vx - a.vg[0]), dY = a.dt * (vy - a.vg[1]), dZ = a.dt * (vz - a.vg[2]);
@@ -299,7 +302,7 @@ __global__ void __launch_bounds__(256) push_stag_kernel(PushArgs a) {
   }
   double ux, uy, uz;
   push_u(a, p, f, ux, uy, uz);
-  const double ig = 1.0 / sqrt(1.0 + (ux * ux + uy * uy + uz * uz) * a.inv_c2);
+  const double ig = rsqrt(1.0 + (ux * ux + uy * uy + uz * uz) * a.inv_c2);
   const double v[3] = {ux * ig, uy * ig, uz * ig};
   double mid[3], nw[3];
 #pragma unroll
@@ -473,13 +476,6 @@ __device__ __forceinline__ bool finite_bits(double v) {
   return ((__double_as_longlong(v) >> 52) & 0x7ff) != 0x7ff;
 }
 __device__ __forceinline__ int exponent_of(double v) { return (int)(__double_as_longlong(v) >> 52) & 0x7ff; }
-
-// x in [0, L) after a move of less than a period: as wrap(), the comparisons on the bit patterns
-__device__ __forceinline__ double wrap_bits(double x, double L) {
-  if (__double_as_longlong(x) >= __double_as_longlong(L)) x -= L;  // x >= L > 0
-  if (__double_as_longlong(x) < 0 && x < 0.0) x += L;
-  return x;
-}
 
 __device__ __forceinline__ void window_add(uint32_t* lo, uint32_t* hi, int64_t c) {
   const uint32_t cl = (uint32_t)c;
@@ -718,7 +714,7 @@ __global__ void __launch_bounds__(kThreads64, 2) push64_tile_kernel(const __grid
     }
     double ux, uy, uz;
     push_u(a, p, f, ux, uy, uz);
-    const double ig = 1.0 / sqrt(1.0 + (ux * ux + uy * uy + uz * uz) * a.inv_c2);
+    const double ig = rsqrt(1.0 + (ux * ux + uy * uy + uz * uz) * a.inv_c2);
     const double v[3] = {ux * ig, uy * ig, uz * ig};
     int64_t* st = t.stash + slot;
     double nx[3];
@@ -727,8 +723,8 @@ __global__ void __launch_bounds__(kThreads64, 2) push64_tile_kernel(const __grid
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const double dd = a.dt * (v[c] - a.vg[c]);
-      const double mx = wrap_bits(x[c] + 0.5 * dd, a.L[c]);
-      nx[c] = wrap_bits(x[c] + dd, a.L[c]);
+      const double mx = wrap(x[c] + 0.5 * dd, a.L[c]);
+      nx[c] = wrap(x[c] + dd, a.L[c]);
       int b;
       int64_t fr;
       in = in && split56<P>(mx, a.inv_dx[c], b, fr);
