@@ -136,7 +136,7 @@ void pic_destroy(pic_ctx* ctx) {
                   ctx->rhoh[0], ctx->Jh, ctx->G, ctx->nodal, ctx->Jn, ctx->bin_tid, ctx->bin_counts,
                   ctx->bin_cursor, ctx->bin_tmp, ctx->cell_counts, ctx->cell_cursor, ctx->adj_work, ctx->bin_gate,
                   ctx->bin_outside, ctx->flt1d, ctx->bin_flags, ctx->k1d32, ctx->flt32, ctx->coefq,
-                  ctx->coefq32, ctx->frame, ctx->dhist, ctx->dev_err, ctx->t64_int, ctx->t64_stash};
+                  ctx->coefq32, ctx->frame, ctx->dhist, ctx->dev_err, ctx->t64_int, ctx->t64_stash, ctx->bin2};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (int q = 0; q < PIC_MAX_BINNED_SPECIES; ++q) {
@@ -144,6 +144,7 @@ void pic_destroy(pic_ctx* ctx) {
     if (ctx->sp_chunk[q]) cudaFree(ctx->sp_chunk[q]);
   }
   for (int q = 0; q < ctx->t64_nold; ++q) cudaFree(ctx->t64_old[q]);
+  for (int q = 0; q < ctx->bin2_nold; ++q) cudaFree(ctx->bin2_old[q]);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
   if (ctx->aux) cudaStreamDestroy(ctx->aux);

@@ -3,6 +3,8 @@
 // FP64, so an FP32 context uses the first half of each).
 #include "pic_internal.cuh"
 
+#include <algorithm>
+
 namespace {
 
 #define PIC_TRY32(x)               \
@@ -211,8 +213,6 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
   for (int c = 0; c < 6; ++c) nodal6[c] = nodal(ctx) + c * nc;
   const bool stag = ctx->cycle == PIC_CYCLE_STAGGERED;
   const bool tiled = ctx->sort_interval > 0 && tiled_push_fits(ctx) && !stag;
-  int64_t total = 0;
-  for (int q = 0; q < n_species; ++q) total += sp[q].n;
   if (tiled) {
     // device scratch of the binning (allocated once; no allocation happens inside the steps)
     if (!ctx->bin_gate) {
@@ -237,10 +237,14 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
       ctx->sp_off_n[q] = sp[q].n;
     }
   }
-  // The first step's (forced) binning of species 0 reads the particles only: it runs on the
+  // The first step's (forced) binning reads the particles only: it runs on the
   // context's second stream, concurrently with the entry transforms of the fields on this one,
   // and the first push waits for it (fork / join by events, also valid inside graph capture).
+  // The one-level binning of large tiles leaves a species' sorted copy in scratch that all share, so
+  // there only species 0 is binned early and the others right before their pushes.
   const bool early_bin = tiled && n_species > 0;
+  const int nbin = std::min(n_species, PIC_MAX_BINNED_SPECIES);
+  const bool two_level = bin32_two_level(ctx), home = ctx->shape_order == 2 && two_level;
   if (early_bin) {
     PIC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
     PIC_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
@@ -248,12 +252,11 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
     ctx->stream = ctx->aux;
     pic_status st = PIC_OK;
     {
-      StageScope t(ctx, STAGE_BIN, 1);
-      st = particles_bin32_decide(ctx, total, 1);
-    }
-    if (st == PIC_OK) {
-      StageScope t(ctx, STAGE_BIN, bin32_launches(ctx, sp[0].n, true, false));
-      st = particles_bin32(ctx, &sp[0], ctx->sp_off[0], ctx->bin_gate, ctx->sp_chunk[0], false, ctx->frame);
+      StageScope t(ctx, STAGE_BIN, 1 + bin32_launches(ctx, sp, two_level ? nbin : 1));
+      st = particles_begin32(ctx, sp, n_species, false, true, true, nullptr, nullptr);
+      if (st == PIC_OK)
+        st = two_level ? particles_bin32_step(ctx, sp, nbin, ctx->sp_off, ctx->sp_chunk, ctx->bin_gate, ctx->frame, home)
+                       : particles_bin32(ctx, &sp[0], ctx->sp_off[0], ctx->bin_gate, ctx->sp_chunk[0], false, ctx->frame);
     }
     ctx->stream = main_stream;
     if (st != PIC_OK) return st;
@@ -299,23 +302,26 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
     // when the previous push moved more than 2 % of the particles out of their tile (they would
     // gather from global memory in the next push).
     if (tiled) {
-      const int force = (s == 0 || since_forced >= ctx->sort_interval) ? 1 : 0;
+      const bool force = s == 0 || since_forced >= ctx->sort_interval;
       since_forced = force ? 1 : since_forced + 1;
-      if (!(s == 0 && early_bin)) {  // step 0: decided on the second stream
-        StageScope t(ctx, STAGE_BIN, 1);
-        PIC_TRY32(particles_bin32_decide(ctx, total, force));
-      }
+      // also clears J and rho; after the first step the tile frames follow the species' drift (binning
+      // stays off while they keep their tiles).  Step 0 is decided (and binned) on the second stream.
+      const bool first = s == 0 && early_bin;
+      StageScope t(ctx, STAGE_BIN, 1 + (first || !two_level ? 0 : bin32_launches(ctx, sp, nbin)));
+      PIC_TRY32(particles_begin32(ctx, sp, n_species, s > 0, !first, force, jn, rho));
+      if (first) PIC_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
+      else if (two_level && nbin > 0)
+        PIC_TRY32(particles_bin32_step(ctx, sp, nbin, ctx->sp_off, ctx->sp_chunk, ctx->bin_gate, ctx->frame, home));
+    } else {
+      PIC_CUDA_TRY(ctx, cudaMemsetAsync(jn, 0, 3 * nc * sizeof(float), ctx->stream));
+      PIC_CUDA_TRY(ctx, cudaMemsetAsync(rho, 0, nc * sizeof(float), ctx->stream));
     }
-    PIC_CUDA_TRY(ctx, cudaMemsetAsync(jn, 0, 3 * nc * sizeof(float), ctx->stream));
-    PIC_CUDA_TRY(ctx, cudaMemsetAsync(rho, 0, nc * sizeof(float), ctx->stream));
     for (int q = 0; q < n_species; ++q) {
       if (tiled && q < PIC_MAX_BINNED_SPECIES) {
-        // the binning leaves the sorted species in the shared scratch and the push copies it back
-        // (so each species is binned right before its own push)
-        if (s == 0 && q == 0 && early_bin) {
-          PIC_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));  // binned on the second stream
-        } else {
-          StageScope t(ctx, STAGE_BIN, bin32_launches(ctx, sp[q].n, true, false));
+        // (large tiles) the binning leaves the sorted species in the shared scratch and the push copies
+        // it back, so each species is binned right before its own push
+        if (!two_level && !(s == 0 && q == 0)) {
+          StageScope t(ctx, STAGE_BIN, bin32_launches(ctx, &sp[q], 1));
           PIC_TRY32(particles_bin32(ctx, &sp[q], ctx->sp_off[q], ctx->bin_gate, ctx->sp_chunk[q], false,
                                     ctx->frame + 8 * q));
         }
@@ -323,17 +329,17 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
         // works, its twin returns
         StageScope t(ctx, STAGE_PUSH, sp[q].n > 0 ? (ctx->vg[2] != 0.0 ? 2 : 1) : 0);
         PIC_TRY32(particles_push32_tiled(ctx, En, Bn, &sp[q], Jnp, rho, ctx->sp_off[q], ctx->sp_chunk[q],
-                                         bin32_two_level(ctx) ? nullptr : bin32_scatter_gate(ctx),
+                                         two_level ? nullptr : bin32_scatter_gate(ctx),
                                          ctx->frame + 8 * q, ctx->dhist + 10 * q));
       } else {
         StageScope t(ctx, STAGE_PUSH, sp[q].n > 0 ? 1 : 0);
         PIC_TRY32(particles_push32(ctx, En, Bn, &sp[q], Jnp, rho));
       }
     }
-    if (tiled) {
-      // the tile frames follow the species' drift (binning stays off while they keep their tiles)
+    if (tiled && last && n_species > 0) {
+      // the frames of the next call's species
       StageScope t(ctx, STAGE_BIN, 1);
-      PIC_TRY32(particles_frames_advance(ctx, sp, n_species));
+      PIC_TRY32(particles_begin32(ctx, sp, n_species, true, false, false, nullptr, nullptr));
     }
     if (fd) {
       // J^{n+1/2}: optional smoothing, nodes -> Yee (work arrays: the nodal E, B, free after the

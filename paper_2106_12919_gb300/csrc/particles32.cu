@@ -265,6 +265,12 @@ __device__ __forceinline__ int shape_base_offset(float f) {
   return P == 2 ? (f >= 0.5f ? 0 : -1) : (P == 3 ? -1 : 0);
 }
 
+// the home of a particle of cell i: the node its tile and place are chosen by (see Key32Args::home)
+template <int P>
+__device__ __forceinline__ int home_offset(float f) {
+  return P == 2 && f >= 0.5f ? 1 : 0;
+}
+
 // J of one particle (cell (ix, iy, iz) + offsets: the current-deposit midpoint) over NS + 1 z nodes
 // from node lz0, its own block starting lz - lz0 = 0 or 1 nodes in and the other node taking 0; a
 // particle whose block starts elsewhere, or that leaves the window, deposits through global
@@ -563,8 +569,9 @@ __device__ __forceinline__ void deposit_phase(const Push32Args& a, const Window&
     const int mx = nx + move_offset(nfx, hX, mfx), my = ny + move_offset(nfy, hY, mfy),
               mz = nz + move_offset(nfz, hZ, mfz);
     if (JEXT) {
-      const int ozmin = __reduce_min_sync(__activemask(), mz - nz + shape_base_offset<P>(mfz));
-      deposit_j5<P>(a, win, mx, my, mz, mfx, mfy, mfz, qw * vx, qw * vy, qw * vz, nz + ozmin);
+      const int hz = nz + home_offset<P>(nfz);  // lanes are spread over their homes
+      const int ozmin = __reduce_min_sync(__activemask(), mz - hz + shape_base_offset<P>(mfz));
+      deposit_j5<P>(a, win, mx, my, mz, mfx, mfy, mfz, qw * vx, qw * vy, qw * vz, hz + ozmin);
     } else {
       deposit_window<P>(a, win, mx, my, mz, mfx, mfy, mfz, qw * vx, qw * vy, qw * vz, 0.f, true);
     }
@@ -745,15 +752,17 @@ __global__ void __launch_bounds__(kTileThreads, 1024 / kTileThreads) push32_tile
     const int nx = ix + move_offset(fx, dX, nfx), ny = iy + move_offset(fy, dY, nfy),
               nz = iz + move_offset(fz, dZ, nfz);
     // the next push gathers this particle from the staged nodes of this tile only while its new
-    // cell stays in the tile: count those that leave (the device re-bins before the next push
+    // home stays in the tile: count those that leave (the device re-bins before the next push
     // when they exceed 2 % of all particles)
-    nout += (((nx - s_next[0]) & a.mask[0]) >= t.T[0] || ((ny - s_next[1]) & a.mask[1]) >= t.T[1] ||
-             ((nz - s_next[2]) & a.mask[2]) >= t.T[2])
+    const int hx = nx + home_offset<P>(nfx), hy = ny + home_offset<P>(nfy), hz = nz + home_offset<P>(nfz);
+    nout += (((hx - s_next[0]) & a.mask[0]) >= t.T[0] || ((hy - s_next[1]) & a.mask[1]) >= t.T[1] ||
+             ((hz - s_next[2]) & a.mask[2]) >= t.T[2])
                 ? 1u
                 : 0u;
-    // cell displacements -1 and +1 per axis (the frame velocity estimate of the next step)
-    dpk += (nx - ix == -1 ? 1u : 0u) + (nx - ix == 1 ? 1u << 5 : 0u) + (ny - iy == -1 ? 1u << 10 : 0u) +
-           (ny - iy == 1 ? 1u << 15 : 0u) + (nz - iz == -1 ? 1u << 20 : 0u) + (nz - iz == 1 ? 1u << 25 : 0u);
+    // displacements -1 and +1 of the home per axis (the frame velocity estimate of the next step)
+    const int sx = hx - ix - home_offset<P>(fx), sy = hy - iy - home_offset<P>(fy), sz = hz - iz - home_offset<P>(fz);
+    dpk += (sx == -1 ? 1u : 0u) + (sx == 1 ? 1u << 5 : 0u) + (sy == -1 ? 1u << 10 : 0u) + (sy == 1 ? 1u << 15 : 0u) +
+           (sz == -1 ? 1u << 20 : 0u) + (sz == 1 ? 1u << 25 : 0u);
     a.cell[p] = (((nx & a.mask[0]) * (int)a.Ny + (ny & a.mask[1])) * (int)a.Nz) + (nz & a.mask[2]);
     a.fx[p] = nfx;
     a.fy[p] = nfy;
@@ -1043,36 +1052,52 @@ __global__ void scatter_gate_kernel(const int* gate, const int* unsorted, int* s
   *sgate = ((gate == nullptr || *gate != 0) && *unsorted != 0) ? 1 : 0;
 }
 
-// gate = (particles whose new cell left their tile in the last push) > limit, or forced; resets the count
-__global__ void bin_decide_kernel(int* gate, unsigned long long* outside, unsigned long long limit, int force) {
-  *gate = (force || *outside > limit) ? 1 : 0;
-  *outside = 0ull;
-}
-
-struct FrameArgs {
+// What a step of the tiled form does before its binning, in one launch.  Each part is optional.
+//  - advance: after a push, every binned species' tile frame moves by the velocity that push assumed;
+//    the new velocity is the displacement that at least 3/4 of the species' particles made (else 0)
+//  - decide: gate = (particles whose new cell left their tile in the last push) > limit, or forced;
+//    resets the count
+//  - zero: clears the nodal J and rho of the step's deposits
+struct Begin32Args {
+  int advance, decide, force;
+  int* gate;
+  unsigned long long* outside;
+  unsigned long long limit;
   int* frame;                 // + 8 q: shift [0..2], velocity [4..6]
   unsigned long long* dhist;  // + 10 q: counts of displacements -1, +1 for x, y, z
   int64_t n[PIC_MAX_BINNED_SPECIES];
   int mask[3];
   int nsp;
+  float2 *zero_j, *zero_rho;  // or null
+  int64_t nj, nrho;           // pairs of floats
 };
 
-// one thread per species: the frame moves by the velocity the last push assumed; the new velocity
-// is the displacement at least 3/4 of the species' particles made (else 0)
-__global__ void frames_advance_kernel(FrameArgs a) {
-  const int q = threadIdx.x;
-  if (q >= a.nsp) return;
-  int* f = a.frame + 8 * q;
-  unsigned long long* h = a.dhist + 10 * q;
-  const unsigned long long n = (unsigned long long)a.n[q];
+__global__ void __launch_bounds__(256) begin32_kernel(Begin32Args a) {
+  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+  if (blockIdx.x == 0) {
+    const int q = threadIdx.x;
+    if (a.advance && q < a.nsp) {
+      int* f = a.frame + 8 * q;
+      unsigned long long* h = a.dhist + 10 * q;
+      const unsigned long long n = (unsigned long long)a.n[q];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    f[d] = (f[d] + f[4 + d]) & a.mask[d];
-    const unsigned long long neg = h[2 * d], pos = h[2 * d + 1];
-    f[4 + d] = (n > 0 && 4 * neg >= 3 * n) ? -1 : ((n > 0 && 4 * pos >= 3 * n) ? 1 : 0);
-    h[2 * d] = 0ull;
-    h[2 * d + 1] = 0ull;
+      for (int d = 0; d < 3; ++d) {
+        f[d] = (f[d] + f[4 + d]) & a.mask[d];
+        const unsigned long long neg = h[2 * d], pos = h[2 * d + 1];
+        f[4 + d] = (n > 0 && 4 * neg >= 3 * n) ? -1 : ((n > 0 && 4 * pos >= 3 * n) ? 1 : 0);
+        h[2 * d] = 0ull;
+        h[2 * d + 1] = 0ull;
+      }
+    }
+    if (a.decide && q == 32) {
+      *a.gate = (a.force || *a.outside > a.limit) ? 1 : 0;
+      *a.outside = 0ull;
+    }
   }
+  if (a.zero_j)
+    for (int64_t e = t0; e < a.nj / 2; e += nt) reinterpret_cast<float4*>(a.zero_j)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (a.zero_rho)  // (the caller's array: 8-byte aligned)
+    for (int64_t e = t0; e < a.nrho; e += nt) a.zero_rho[e] = make_float2(0.f, 0.f);
 }
 
 struct Key32Args {
@@ -1091,6 +1116,12 @@ struct Key32Args {
   int* unsorted;           // set to 1 when some key is smaller than its predecessor's
   const int* frame;        // the species' tile frame (shift at [0..2]) or null
   int sh[3];               // its shift, loaded by each kernel (load_frame)
+  // Key by the home node instead of the cell: the nearest node (offset >= 1/2: the cell's upper one),
+  // the centre of a quadratic shape block.  With particles of one cell on either of its two nodes the
+  // lanes of a warp start their blocks at random one node apart, and 15 of the quadratic push's 25
+  // shared-memory wavefronts per particle were bank conflicts.
+  int home;
+  const float* off[3];     // offsets in the cell (home only)
 };
 
 // the tile frame's shift into the kernel's copy of the arguments (0 without a frame)
@@ -1101,13 +1132,19 @@ __device__ __forceinline__ Key32Args load_frame(const Key32Args& a) {
   return k;
 }
 
-// key of a cell: tile of the cell shifted by -sh (the tile frame), then the local cell inside it
-__device__ __forceinline__ int key_of(const Key32Args& a, int c) {
-  const int cx = ((c >> (a.shz + a.shy)) - a.sh[0]) & a.mask[0], cy = ((c >> a.shz) - a.sh[1]) & a.mask[1],
-            cz = (c - a.sh[2]) & a.mask[2];
+// key of a cell: tile of the cell shifted by -sh (the tile frame), then the local cell inside it; hx,
+// hy, hz: 1 to take the next cell (home)
+__device__ __forceinline__ int key_of(const Key32Args& a, int c, int hx = 0, int hy = 0, int hz = 0) {
+  const int cx = ((c >> (a.shz + a.shy)) + hx - a.sh[0]) & a.mask[0], cy = ((c >> a.shz) + hy - a.sh[1]) & a.mask[1],
+            cz = (c + hz - a.sh[2]) & a.mask[2];
   const int t = (int)(((cx >> a.tshift[0]) * a.nty + (cy >> a.tshift[1])) * a.ntz + (cz >> a.tshift[2]));
   const int local = ((((cy & a.tmask[1]) << a.lshift_x) | (cx & a.tmask[0])) << a.lshift_z) | (cz & a.tmask[2]);
   return (t << a.cpt_shift) | local;
+}
+
+__device__ __forceinline__ int key_at(const Key32Args& a, int64_t p) {
+  const int c = a.cell[p];
+  return a.home ? key_of(a, c, a.off[0][p] >= 0.5f, a.off[1][p] >= 0.5f, a.off[2][p] >= 0.5f) : key_of(a, c);
 }
 
 __device__ __forceinline__ bool key32_one(const Key32Args& a, int64_t p) {
@@ -1314,17 +1351,26 @@ __global__ void copy_back_kernel(CopyBackArgs a) {
 constexpr int kMaxLocalCells = 4096;
 constexpr int kOrderThreads = 256;
 
+// The four kernels of a binning: counts and keys out of order, scans and chunk lists, grouping by tile,
+// order inside the tiles.  They run every step and return at once while the gate is off; the first two
+// take every species in one launch.  (They were 15 launches per species, with the gate, frame and
+// clearing launches 20 per step: half of the time of a small step.)
+struct BinBatch {
+  Key32Args k[PIC_MAX_BINNED_SPECIES];
+  const int* gate;
+};
+
 // per particle: key (sortedness check against its predecessor) and the tile histogram
-__global__ void tile_count_kernel(Key32Args a0) {
-  if (gated_off(a0.gate)) return;
-  const Key32Args a = load_frame(a0);
+__global__ void tile_count_kernel(BinBatch b) {
+  if (gated_off(b.gate)) return;
+  const Key32Args a = load_frame(b.k[blockIdx.y]);
   bool mine = false;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < a.n; p += (int64_t)gridDim.x * blockDim.x) {
-    const int k = key_of(a, a.cell[p]);
+    const int k = key_at(a, p);
     const unsigned active = __activemask();
     const int lane_id = threadIdx.x & 31;
     const int up = __shfl_up_sync(active, k, 1);
-    const int prev = lane_id > 0 ? up : (p > 0 ? key_of(a, a.cell[p - 1]) : k);
+    const int prev = lane_id > 0 ? up : (p > 0 ? key_at(a, p - 1) : k);
     mine |= prev > k;
     const int t = k >> a.cpt_shift;
     const unsigned peers = __match_any_sync(active, t);
@@ -1333,20 +1379,133 @@ __global__ void tile_count_kernel(Key32Args a0) {
   flag_unsorted(a, mine);
 }
 
-struct TileScatterArgs {
+struct BinScan {
   const int* gate;
+  int n_tiles;
+  uint32_t* counts[PIC_MAX_BINNED_SPECIES];  // [n_tiles], cleared after use for the next binning
+  uint32_t* cursor[PIC_MAX_BINNED_SPECIES];  // [n_tiles]: first place of each tile
+  int64_t* off[PIC_MAX_BINNED_SPECIES];      // [n_tiles + 1]
+  uint32_t* chunk[PIC_MAX_BINNED_SPECIES];   // chunk starts [n_tiles + 1] or null
+  uint32_t* cmap[PIC_MAX_BINNED_SPECIES];    // tile of each chunk
+  int* flags;                                // + 2 q: keys out of order (cleared after use), scatter gate
+};
+
+// inclusive sum over the CTA's 1024 threads of a pair; red: 32 pairs
+__device__ __forceinline__ uint2 block_scan_pair(uint2 v, uint2* red) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t x = __shfl_up_sync(0xffffffffu, v.x, o), y = __shfl_up_sync(0xffffffffu, v.y, o);
+    if (lane >= o) v.x += x, v.y += y;
+  }
+  __syncthreads();  // red of the previous call is consumed
+  if (lane == 31) red[wid] = v;
+  __syncthreads();
+  if (wid == 0) {
+    uint2 r = red[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xffffffffu, r.x, o), y = __shfl_up_sync(0xffffffffu, r.y, o);
+      if (lane >= o) r.x += x, r.y += y;
+    }
+    red[lane] = r;
+  }
+  __syncthreads();
+  if (wid > 0) v.x += red[wid - 1].x, v.y += red[wid - 1].y;
+  return v;
+}
+
+// one CTA per species: exclusive scans of the tiles' particle and chunk counts (4 tiles per thread and
+// pass), the tile of every chunk, and the scatter gate (an already ordered species needs its tile ranges
+// but no permutation)
+__global__ void __launch_bounds__(1024) bin_scan_kernel(BinScan a) {
+  if (gated_off(a.gate)) return;
+  __shared__ uint2 red[32];
+  const int q = blockIdx.x;
+  uint32_t* counts = a.counts[q];
+  uint32_t* cursor = a.cursor[q];
+  int64_t* off = a.off[q];
+  uint32_t* chunk = a.chunk[q];
+  uint32_t* cmap = a.cmap[q];
+  uint2 base = make_uint2(0u, 0u);
+  for (int t0 = 0; t0 < a.n_tiles; t0 += 4096) {
+    uint32_t n[4], c[4];
+    uint2 s = make_uint2(0u, 0u);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int t = t0 + 4 * threadIdx.x + e;
+      n[e] = t < a.n_tiles ? counts[t] : 0u;
+      c[e] = (n[e] + kTileChunk - 1) / kTileChunk;
+      s.x += n[e];
+      s.y += c[e];
+    }
+    const uint2 inc = block_scan_pair(s, red);
+    uint2 run = make_uint2(base.x + inc.x - s.x, base.y + inc.y - s.y);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int t = t0 + 4 * threadIdx.x + e;
+      if (t < a.n_tiles) {
+        counts[t] = 0u;
+        cursor[t] = run.x;
+        off[t] = (int64_t)run.x;
+        if (chunk) {
+          chunk[t] = run.y;
+          for (uint32_t k = 0; k < c[e]; ++k) cmap[run.y + k] = (uint32_t)t;
+        }
+      }
+      run.x += n[e];
+      run.y += c[e];
+    }
+    base.x += red[31].x;
+    base.y += red[31].y;
+  }
+  if (threadIdx.x == 0) {
+    off[a.n_tiles] = (int64_t)base.x;
+    if (chunk) chunk[a.n_tiles] = base.y;
+    a.flags[2 * q + 1] = a.flags[2 * q] != 0 ? 1 : 0;
+    a.flags[2 * q] = 0;
+  }
+}
+
+// after the multi-kernel scan (see particles_bin32): the offsets, scanned in place, become the cursors
+__global__ void scan_finish_kernel(uint32_t* counts, uint32_t* cursor, int64_t n, int* flags, const int* gate) {
+  if (gated_off(gate)) return;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+    cursor[t] = counts[t];
+    counts[t] = 0u;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    flags[1] = flags[0] != 0 ? 1 : 0;
+    flags[0] = 0;
+  }
+}
+
+struct TileScatterArgs {
+  const int* gate;                 // the binning's gate; off: the scatter gate of this binning is stale
+  const int* sgate;                // the species' scatter gate
   Key32Args k;
   uint32_t* spc[8];                // the species arrays: cell, fx, fy, fz, ux, uy, uz, w as 32-bit words
   uint32_t* tmp[8];                // scratch of the same layout
   unsigned long long* id_spc;      // optional ids
   unsigned long long* id_tmp;
-  const uint32_t* off;             // exclusive tile offsets
-  uint32_t* cursor;                // zeroed, per tile
+  uint32_t* cursor;                // per tile: its next free place
 };
+
+// key of a particle given as its words, and of particle j of the scratch
+__device__ __forceinline__ int word_key(const Key32Args& k, const uint32_t* v) {
+  return k.home ? key_of(k, (int)v[0], __uint_as_float(v[1]) >= 0.5f, __uint_as_float(v[2]) >= 0.5f,
+                         __uint_as_float(v[3]) >= 0.5f)
+                : key_of(k, (int)v[0]);
+}
+__device__ __forceinline__ int tmp_key(const TileScatterArgs& a, int64_t j) {
+  const uint32_t v[4] = {a.tmp[0][j], a.k.home ? a.tmp[1][j] : 0u, a.k.home ? a.tmp[2][j] : 0u,
+                         a.k.home ? a.tmp[3][j] : 0u};
+  return word_key(a.k, v);
+}
 
 // level 1: species arrays -> scratch, grouped by tile (order inside a tile: arbitrary)
 __global__ void tile_scatter_kernel(TileScatterArgs a) {
-  if (gated_off(a.gate)) return;
+  if (gated_off(a.gate) || *a.sgate == 0) return;
   a.k = load_frame(a.k);
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < a.k.n; p += (int64_t)gridDim.x * blockDim.x) {
     // the particle's words are loaded before the cursor atomic (which the compiler may not move
@@ -1355,7 +1514,7 @@ __global__ void tile_scatter_kernel(TileScatterArgs a) {
 #pragma unroll
     for (int f = 0; f < 8; ++f) v[f] = a.spc[f][p];
     const unsigned long long id = a.id_spc ? a.id_spc[p] : 0ull;
-    const int t = key_of(a.k, (int)v[0]) >> a.k.cpt_shift;
+    const int t = word_key(a.k, v) >> a.k.cpt_shift;
     const unsigned active = __activemask();
     const unsigned peers = __match_any_sync(active, t);
     const int lane = threadIdx.x & 31;
@@ -1364,7 +1523,7 @@ __global__ void tile_scatter_kernel(TileScatterArgs a) {
     uint32_t base = 0;
     if (lane == leader) base = atomicAdd(a.cursor + t, (uint32_t)__popc(peers));
     base = __shfl_sync(peers, base, leader);
-    const int64_t q = (int64_t)a.off[t] + base + rank;
+    const int64_t q = (int64_t)base + rank;
 #pragma unroll
     for (int f = 0; f < 8; ++f) a.tmp[f][q] = v[f];
     if (a.id_spc) a.id_tmp[q] = id;
@@ -1373,13 +1532,18 @@ __global__ void tile_scatter_kernel(TileScatterArgs a) {
 
 // level 2: scratch -> species arrays, each tile ordered by local cell: one CTA per tile (grid-stride
 // over the tiles), a shared-memory counting sort (the order among the particles of one cell is
-// that of the shared-memory atomics, i.e. unspecified)
+// that of the shared-memory atomics, i.e. unspecified).  Tiles of up to kMaxOrder particles list the
+// sorted order in shared memory and read the scratch through it: the reads stay within the tile's few
+// kilobytes per array (L1), and the writes are whole lines, where writing each particle to its place
+// sent 4-byte pieces of a line to L2 one by one (larger tiles still do).
+constexpr int kMaxOrder = 4096;
 __global__ void __launch_bounds__(kOrderThreads) cell_order_kernel(TileScatterArgs a, const int64_t* tile_off,
                                                                    int64_t n_tiles) {
-  if (gated_off(a.gate)) return;
+  if (gated_off(a.gate) || *a.sgate == 0) return;
   a.k = load_frame(a.k);
   __shared__ uint32_t cnt[kMaxLocalCells];
   __shared__ uint32_t part[kOrderThreads];
+  __shared__ uint16_t order[kMaxOrder];
   const int cpt = 1 << a.k.cpt_shift;
   const int lmask = cpt - 1;
   for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
@@ -1387,8 +1551,7 @@ __global__ void __launch_bounds__(kOrderThreads) cell_order_kernel(TileScatterAr
     if (nt == 0) continue;  // uniform over the CTA
     for (int i = threadIdx.x; i < cpt; i += blockDim.x) cnt[i] = 0u;
     __syncthreads();
-    for (int64_t i = threadIdx.x; i < nt; i += blockDim.x)
-      atomicAdd(&cnt[key_of(a.k, (int)a.tmp[0][b0 + i]) & lmask], 1u);
+    for (int64_t i = threadIdx.x; i < nt; i += blockDim.x) atomicAdd(&cnt[tmp_key(a, b0 + i) & lmask], 1u);
     __syncthreads();
     // exclusive scan of cnt[0..cpt): each thread a run of cpt / blockDim entries
     const int per = (cpt + blockDim.x - 1) / blockDim.x;
@@ -1410,19 +1573,34 @@ __global__ void __launch_bounds__(kOrderThreads) cell_order_kernel(TileScatterAr
       run += c;
     }
     __syncthreads();
-    for (int64_t i = threadIdx.x; i < nt; i += blockDim.x) {
-      const int64_t j = b0 + i;
-      uint32_t v[8];
+    if (nt <= kMaxOrder) {
+      for (int i = threadIdx.x; i < (int)nt; i += blockDim.x)
+        order[atomicAdd(&cnt[tmp_key(a, b0 + i) & lmask], 1u)] = (uint16_t)i;
+      __syncthreads();
+      for (int i = threadIdx.x; i < (int)nt; i += blockDim.x) {
+        const int64_t j = b0 + order[i];
+        uint32_t v[8];
 #pragma unroll
-      for (int f = 0; f < 8; ++f) v[f] = a.tmp[f][j];
-      const unsigned long long id = a.id_spc ? a.id_tmp[j] : 0ull;
-      const int l = key_of(a.k, (int)v[0]) & lmask;
-      const int64_t q = b0 + atomicAdd(&cnt[l], 1u);
+        for (int f = 0; f < 8; ++f) v[f] = a.tmp[f][j];
+        const unsigned long long id = a.id_spc ? a.id_tmp[j] : 0ull;
 #pragma unroll
-      for (int f = 0; f < 8; ++f) a.spc[f][q] = v[f];
-      if (a.id_spc) a.id_spc[q] = id;
+        for (int f = 0; f < 8; ++f) a.spc[f][b0 + i] = v[f];
+        if (a.id_spc) a.id_spc[b0 + i] = id;
+      }
+    } else {
+      for (int64_t i = threadIdx.x; i < nt; i += blockDim.x) {
+        const int64_t j = b0 + i;
+        uint32_t v[8];
+#pragma unroll
+        for (int f = 0; f < 8; ++f) v[f] = a.tmp[f][j];
+        const unsigned long long id = a.id_spc ? a.id_tmp[j] : 0ull;
+        const int64_t q = b0 + atomicAdd(&cnt[word_key(a.k, v) & lmask], 1u);
+#pragma unroll
+        for (int f = 0; f < 8; ++f) a.spc[f][q] = v[f];
+        if (a.id_spc) a.id_spc[q] = id;
+      }
     }
-    __syncthreads();  // cnt is reused by the next tile
+    __syncthreads();  // cnt and order are reused by the next tile
   }
 }
 
@@ -1432,22 +1610,29 @@ __global__ void __launch_bounds__(kOrderThreads) cell_order_kernel(TileScatterAr
 #define PIC_BIN_LIMIT 0.02
 #endif
 
-pic_status particles_bin32_decide(pic_ctx* ctx, int64_t total_particles, int force) {
-  const unsigned long long limit = (unsigned long long)(PIC_BIN_LIMIT * (double)total_particles);
-  bin_decide_kernel<<<1, 1, 0, ctx->stream>>>(ctx->bin_gate, ctx->bin_outside, limit, force);
-  PIC_LAUNCH_CHECK(ctx);
-  return PIC_OK;
-}
-
-pic_status particles_frames_advance(pic_ctx* ctx, const pic_species32* sp, int n_species) {
-  FrameArgs f;
-  f.frame = ctx->frame;
-  f.dhist = ctx->dhist;
-  f.nsp = std::min(n_species, PIC_MAX_BINNED_SPECIES);
-  for (int q = 0; q < PIC_MAX_BINNED_SPECIES; ++q) f.n[q] = q < f.nsp ? sp[q].n : 0;
-  for (int d = 0; d < 3; ++d) f.mask[d] = (int)ctx->N[d] - 1;
-  if (f.nsp <= 0 || !ctx->frame) return PIC_OK;
-  frames_advance_kernel<<<1, 32, 0, ctx->stream>>>(f);
+pic_status particles_begin32(pic_ctx* ctx, const pic_species32* sp, int n_species, bool advance, bool decide, bool force,
+                             float* zero_j, float* zero_rho) {
+  Begin32Args a;
+  memset(&a, 0, sizeof(a));
+  a.advance = advance ? 1 : 0;
+  a.decide = decide ? 1 : 0;
+  a.force = force ? 1 : 0;
+  a.gate = ctx->bin_gate;
+  a.outside = ctx->bin_outside;
+  a.frame = ctx->frame;
+  a.dhist = ctx->dhist;
+  a.nsp = std::min(n_species, PIC_MAX_BINNED_SPECIES);
+  int64_t total = 0;
+  for (int q = 0; q < n_species; ++q) total += sp[q].n;
+  for (int q = 0; q < a.nsp; ++q) a.n[q] = sp[q].n;
+  a.limit = (unsigned long long)(PIC_BIN_LIMIT * (double)total);
+  for (int d = 0; d < 3; ++d) a.mask[d] = (int)ctx->N[d] - 1;
+  a.zero_j = reinterpret_cast<float2*>(zero_j);
+  a.zero_rho = reinterpret_cast<float2*>(zero_rho);
+  a.nj = 3 * ctx->ncell / 2;
+  a.nrho = ctx->ncell / 2;
+  const int64_t want = zero_j ? (ctx->ncell + 1023) / 1024 : 1;
+  begin32_kernel<<<(unsigned)std::min<int64_t>(want, 152 * 8), 256, 0, ctx->stream>>>(a);
   PIC_LAUNCH_CHECK(ctx);
   return PIC_OK;
 }
@@ -1469,12 +1654,20 @@ bool bin32_two_level(const pic_ctx* ctx) {
   return int64_t(ctx->tile[0]) * ctx->tile[1] * ctx->tile[2] <= kMaxLocalCells;
 }
 
-int bin32_launches(const pic_ctx* ctx, int64_t n, bool chunks, bool copy_back) {
-  // fill, (count), three scan kernels, (five chunk-list kernels), then for n > 0 the scatter gate,
-  // the cursor fill and the scatter (and the in-tile ordering, or the copy back)
-  const int head = 1 + (n > 0 ? 1 : 0) + 3 + (chunks ? 5 : 0);
-  if (n == 0) return head;
-  return head + 3 + ((bin32_two_level(ctx) || copy_back) ? 1 : 0);
+// tiles up to which one CTA scans a species' counts (4096 per pass, about 1 us each)
+constexpr int64_t kMaxScanTiles = 1 << 17;
+
+int bin32_launches(const pic_ctx* ctx, const pic_species32* sp, int n_species) {
+  if (!bin32_two_level(ctx)) {
+    // fill, (keys), three scan kernels, five chunk-list kernels, then the scatter gate, the cursor fill
+    // and the scatter
+    int n = 0;
+    for (int q = 0; q < n_species; ++q) n += 9 + (sp[q].n > 0 ? 4 : 0);
+    return n;
+  }
+  int n = 1 + (ctx->n_tiles <= kMaxScanTiles ? 1 : 9 * n_species);
+  for (int q = 0; q < n_species; ++q) n += sp[q].n > 0 ? 2 : 0;
+  return n;
 }
 
 bool tiled_push_fits(const pic_ctx* ctx) {
@@ -1544,25 +1737,12 @@ static pic_status build_chunks(pic_ctx* ctx, const int64_t* tile_off, uint32_t* 
   return PIC_OK;
 }
 
-pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offsets_out, const int* gate,
-                           uint32_t* chunks_out, bool copy_back, const int* frame) {
-  const int64_t n = sp->n;
-  pic_status st = particles_bin_capacity(ctx, n > 0 ? n : 1);
-  if (st != PIC_OK) return st;
-  const int64_t ncell = ctx->ncell;
-  const int64_t nblk = (ncell + kScanBlock - 1) / kScanBlock;
-  if (!ctx->cell_counts) {
-    // counts/offsets per cell, block sums, total
-    PIC_CUDA_TRY(ctx, cudaMalloc(&ctx->cell_counts, (ncell + nblk + 2) * sizeof(uint32_t)));
-  }
-  uint32_t* counts = ctx->cell_counts;
-  uint32_t* bsum = counts + ncell;
-  uint32_t* total = bsum + nblk;
-  const unsigned fill_blocks = 152 * 8;
+// key geometry of one species
+static Key32Args key_args(const pic_ctx* ctx, const pic_species32* sp, const int* frame, bool home) {
   Key32Args b;
-  b.gate = gate;
+  memset(&b, 0, sizeof(b));
   b.cell = sp->cell;
-  b.n = n;
+  b.n = sp->n;
   b.shz = ilog2(ctx->N[2]);
   b.shy = ilog2(ctx->N[1]);
   for (int d = 0; d < 3; ++d) {
@@ -1575,10 +1755,131 @@ pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offse
   b.lshift_x = ilog2(ctx->tile[0]);
   b.lshift_z = ilog2(ctx->tile[2]);
   b.cpt_shift = ilog2(ctx->tile[0]) + ilog2(ctx->tile[1]) + ilog2(ctx->tile[2]);
+  b.frame = frame;
+  b.home = home ? 1 : 0;
+  b.off[0] = sp->fx;
+  b.off[1] = sp->fy;
+  b.off[2] = sp->fz;
+  return b;
+}
+
+// scratch of the two-level binning for nsp species: flags, and per species counts (cleared here, and by
+// every binning after use) and cursors
+static pic_status bin32_scratch(pic_ctx* ctx, int nsp) {
+  if (ctx->bin2_species >= nsp) return PIC_OK;
+  // all of them at the first use, as far as they are few: nothing is allocated between two steps
+  const int want = std::max(nsp, std::min(PIC_MAX_BINNED_SPECIES, 2));
+  uint32_t* w = nullptr;
+  const size_t words = 2 * PIC_MAX_BINNED_SPECIES + (size_t)want * 2 * ctx->n_tiles;
+  if (cudaMalloc(&w, words * sizeof(uint32_t)) != cudaSuccess) {
+    cudaGetLastError();
+    return pic_set_error(ctx, PIC_ERR_NOMEM, "binning scratch");
+  }
+  if (ctx->bin2) {
+    ctx->bin2_old[ctx->bin2_nold++] = ctx->bin2;  // a captured graph may still use it: freed with the context
+  }
+  ctx->bin2 = w;
+  ctx->bin2_species = want;
+  PIC_CUDA_TRY(ctx, cudaMemsetAsync(w, 0, words * sizeof(uint32_t), ctx->stream));
+  return PIC_OK;
+}
+
+pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_species, int64_t* const* offsets,
+                                uint32_t* const* chunks, const int* gate, const int* frames, bool home) {
+  PIC_TRY(bin32_scratch(ctx, n_species));
+  int64_t nmax = 1;
+  for (int q = 0; q < n_species; ++q) nmax = std::max(nmax, sp[q].n);
+  PIC_TRY(particles_bin_capacity(ctx, nmax));
+  const int64_t nt = ctx->n_tiles;
+  int* flags = reinterpret_cast<int*>(ctx->bin2);
+  BinBatch b;
+  BinScan sc;
+  memset(&sc, 0, sizeof(sc));
+  b.gate = sc.gate = gate;
+  sc.n_tiles = (int)nt;
+  sc.flags = flags;
+  for (int q = 0; q < n_species; ++q) {
+    Key32Args& k = b.k[q];
+    k = key_args(ctx, &sp[q], frames ? frames + 8 * q : nullptr, home);
+    k.counts = ctx->bin2 + 2 * PIC_MAX_BINNED_SPECIES + (size_t)q * 2 * nt;
+    k.unsorted = flags + 2 * q;
+    sc.counts[q] = k.counts;
+    sc.cursor[q] = k.counts + nt;
+    sc.off[q] = offsets && offsets[q] ? offsets[q] : ctx->bin_counts;
+    sc.chunk[q] = chunks ? chunks[q] : nullptr;
+    sc.cmap[q] = chunks ? chunks[q] + chunk_map_offset(ctx) : nullptr;
+  }
+  // grid-stride kernels on a capped grid: when the gate is off they return at once
+  const int bs = 256;
+  const auto blocks = [&](int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + bs - 1) / bs, 152 * 8)); };
+  tile_count_kernel<<<dim3(blocks(nmax), (unsigned)n_species), bs, 0, ctx->stream>>>(b);
+  PIC_LAUNCH_CHECK(ctx);
+  if (nt <= kMaxScanTiles) {
+    bin_scan_kernel<<<(unsigned)n_species, 1024, 0, ctx->stream>>>(sc);
+    PIC_LAUNCH_CHECK(ctx);
+  } else {
+    // many small tiles: the scans over several CTAs
+    const int64_t nblk = (nt + kScanBlock - 1) / kScanBlock;
+    if (!ctx->cell_counts) PIC_CUDA_TRY(ctx, cudaMalloc(&ctx->cell_counts, (nblk + 2) * sizeof(uint32_t)));
+    uint32_t* bsum = ctx->cell_counts;
+    uint32_t* total = bsum + nblk;
+    for (int q = 0; q < n_species; ++q) {
+      scan_block_kernel<<<(unsigned)std::min<int64_t>(nblk, 152 * 2), 1024, 0, ctx->stream>>>(sc.counts[q], nt, bsum, gate);
+      PIC_LAUNCH_CHECK(ctx);
+      scan_sums_kernel<<<1, 1024, 0, ctx->stream>>>(bsum, nblk, total, gate);
+      PIC_LAUNCH_CHECK(ctx);
+      scan_add_kernel<<<blocks(nt), 256, 0, ctx->stream>>>(sc.counts[q], nt, bsum, 0, sc.off[q], nt, total, gate);
+      PIC_LAUNCH_CHECK(ctx);
+      if (chunks) PIC_TRY(build_chunks(ctx, sc.off[q], sc.chunk[q], gate));
+      scan_finish_kernel<<<blocks(nt), 256, 0, ctx->stream>>>(sc.counts[q], sc.cursor[q], nt, flags + 2 * q, gate);
+      PIC_LAUNCH_CHECK(ctx);
+    }
+  }
+  uint32_t* tmp = reinterpret_cast<uint32_t*>(ctx->bin_tmp);
+  for (int q = 0; q < n_species; ++q) {
+    if (sp[q].n == 0) continue;
+    TileScatterArgs s;
+    s.gate = gate;
+    s.sgate = flags + 2 * q + 1;
+    s.k = b.k[q];
+    void* fields[8] = {sp[q].cell, sp[q].fx, sp[q].fy, sp[q].fz, sp[q].ux, sp[q].uy, sp[q].uz, sp[q].w};
+    for (int f = 0; f < 8; ++f) {
+      s.spc[f] = static_cast<uint32_t*>(fields[f]);
+      s.tmp[f] = tmp + (int64_t)f * ctx->bin_cap;
+    }
+    s.id_spc = reinterpret_cast<unsigned long long*>(sp[q].id);
+    s.id_tmp = reinterpret_cast<unsigned long long*>(ctx->bin_tmp + 4 * ctx->bin_cap);  // words 8n..10n
+    s.cursor = sc.cursor[q];
+    tile_scatter_kernel<<<blocks(sp[q].n), bs, 0, ctx->stream>>>(s);
+    PIC_LAUNCH_CHECK(ctx);
+    cell_order_kernel<<<(unsigned)std::min<int64_t>(nt, 152 * 8), kOrderThreads, 0, ctx->stream>>>(s, sc.off[q], nt);
+    PIC_LAUNCH_CHECK(ctx);
+  }
+  return PIC_OK;
+}
+
+pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offsets_out, const int* gate,
+                           uint32_t* chunks_out, bool copy_back, const int* frame) {
+  const int64_t n = sp->n;
+  if (bin32_two_level(ctx)) {
+    PIC_TRY(particles_bin_capacity(ctx, 1));  // bin_counts
+    return particles_bin32_step(ctx, sp, 1, &offsets_out, chunks_out ? &chunks_out : nullptr, gate, frame, false);
+  }
+  PIC_TRY(particles_bin_capacity(ctx, n > 0 ? n : 1));
+  const int64_t ncell = ctx->ncell;
+  const int64_t nblk = (ncell + kScanBlock - 1) / kScanBlock;
+  if (!ctx->cell_counts) {
+    // counts/offsets per cell, block sums, total
+    PIC_CUDA_TRY(ctx, cudaMalloc(&ctx->cell_counts, (ncell + nblk + 2) * sizeof(uint32_t)));
+  }
+  uint32_t* counts = ctx->cell_counts;
+  uint32_t* bsum = counts + ncell;
+  uint32_t* total = bsum + nblk;
+  const unsigned fill_blocks = 152 * 8;
+  Key32Args b = key_args(ctx, sp, frame, false);
+  b.gate = gate;
   b.key = ctx->bin_tid;
   b.counts = counts;
-  b.frame = frame;
-  b.sh[0] = b.sh[1] = b.sh[2] = 0;
   if (!ctx->bin_flags) PIC_CUDA_TRY(ctx, cudaMalloc(&ctx->bin_flags, 2 * sizeof(int)));
   int* unsorted = ctx->bin_flags;
   int* sgate = ctx->bin_flags + 1;
@@ -1589,55 +1890,6 @@ pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offse
   const int bs = 256;
   const unsigned nb = (unsigned)std::min<int64_t>((n + bs - 1) / bs, fill_blocks);
   int64_t* tile_off = offsets_out ? offsets_out : ctx->bin_counts;
-  if ((int64_t(1) << b.cpt_shift) <= kMaxLocalCells) {
-    // two-level: counting sort by tile, then by cell inside each tile (see tile_count_kernel)
-    const int64_t nt = ctx->n_tiles;
-    const int64_t nblk_t = (nt + kScanBlock - 1) / kScanBlock;
-    uint32_t* tcnt = counts;           // per tile: counts -> exclusive offsets
-    uint32_t* tbsum = counts + nt;     // scan block sums
-    uint32_t* ttotal = tbsum + nblk_t;
-    fill_u32_kernel<<<fill_blocks, 256, 0, ctx->stream>>>(tcnt, nt, 0u, gate);
-    PIC_LAUNCH_CHECK(ctx);
-    if (n > 0) {
-      tile_count_kernel<<<nb, bs, 0, ctx->stream>>>(b);
-      PIC_LAUNCH_CHECK(ctx);
-    }
-    scan_block_kernel<<<(unsigned)std::min<int64_t>(nblk_t, 152 * 2), 1024, 0, ctx->stream>>>(tcnt, nt, tbsum, gate);
-    PIC_LAUNCH_CHECK(ctx);
-    scan_sums_kernel<<<1, 1024, 0, ctx->stream>>>(tbsum, nblk_t, ttotal, gate);
-    PIC_LAUNCH_CHECK(ctx);
-    scan_add_kernel<<<(unsigned)std::min<int64_t>((nt + 255) / 256, fill_blocks), 256, 0, ctx->stream>>>(
-        tcnt, nt, tbsum, 0, tile_off, nt, ttotal, gate);
-    PIC_LAUNCH_CHECK(ctx);
-    if (chunks_out) PIC_TRY(build_chunks(ctx, tile_off, chunks_out, gate));
-    if (n == 0) {
-      PIC_CUDA_TRY(ctx, cudaMemsetAsync(sgate, 0, sizeof(int), ctx->stream));
-      return PIC_OK;
-    }
-    scatter_gate_kernel<<<1, 1, 0, ctx->stream>>>(gate, unsorted, sgate);
-    PIC_LAUNCH_CHECK(ctx);
-    if (!ctx->cell_cursor) PIC_CUDA_TRY(ctx, cudaMalloc(&ctx->cell_cursor, ncell * sizeof(uint32_t)));
-    fill_u32_kernel<<<fill_blocks, 256, 0, ctx->stream>>>(ctx->cell_cursor, nt, 0u, sgate);
-    PIC_LAUNCH_CHECK(ctx);
-    TileScatterArgs s;
-    s.gate = sgate;
-    s.k = b;
-    void* fields[8] = {sp->cell, sp->fx, sp->fy, sp->fz, sp->ux, sp->uy, sp->uz, sp->w};
-    uint32_t* tmp = reinterpret_cast<uint32_t*>(ctx->bin_tmp);
-    for (int f = 0; f < 8; ++f) {
-      s.spc[f] = static_cast<uint32_t*>(fields[f]);
-      s.tmp[f] = tmp + (int64_t)f * ctx->bin_cap;
-    }
-    s.id_spc = reinterpret_cast<unsigned long long*>(sp->id);
-    s.id_tmp = reinterpret_cast<unsigned long long*>(ctx->bin_tmp + 4 * ctx->bin_cap);  // words 8n..10n
-    s.off = tcnt;
-    s.cursor = ctx->cell_cursor;
-    tile_scatter_kernel<<<nb, bs, 0, ctx->stream>>>(s);
-    PIC_LAUNCH_CHECK(ctx);
-    cell_order_kernel<<<(unsigned)std::min<int64_t>(nt, 152 * 8), kOrderThreads, 0, ctx->stream>>>(s, tile_off, nt);
-    PIC_LAUNCH_CHECK(ctx);
-    return PIC_OK;  // the species arrays hold the binned particles
-  }
   // one level: counting sort by cell in tile-major order over the whole grid
   fill_u32_kernel<<<fill_blocks, 256, 0, ctx->stream>>>(counts, ncell, 0u, gate);
   PIC_LAUNCH_CHECK(ctx);

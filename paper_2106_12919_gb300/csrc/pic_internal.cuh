@@ -152,6 +152,12 @@ struct pic_ctx {
   uint32_t* cell_counts;  // FP32 binning: per-cell counts -> offsets, block sums, total
   uint32_t* cell_cursor;  // FP32 binning: per-cell scatter cursors
   double* adj_work;       // reverse mode: rhobar^n, rhobar^{n+1}, 6 nodal force adjoints
+  // FP32 two-level binning: [8][2] flags (keys out of order, scatter gate), then per species [n_tiles]
+  // counts and [n_tiles] cursors; outgrown ones are freed with the context
+  uint32_t* bin2;
+  int bin2_species;
+  uint32_t* bin2_old[PIC_MAX_BINNED_SPECIES];
+  int bin2_nold;
   int* bin_gate;                    // FP32 form: device flag "re-bin before the next push"
   int* bin_flags;                   // FP32 binning: [0] keys out of order, [1] scatter gate (see below)
   unsigned long long* bin_outside;  // FP32 form: particles whose new cell left their tile in the last push
@@ -387,20 +393,26 @@ pic_status particles_push32_tiled(pic_ctx* ctx, const float* const En[3], const 
 // the cell shifted by -frame[0..2].
 pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offsets_out, const int* gate = nullptr,
                            uint32_t* chunks_out = nullptr, bool copy_back = true, const int* frame = nullptr);
-// *bin_gate = (particles whose new cell left their tile in the last tiled push > 2 % of total) || force
-pic_status particles_bin32_decide(pic_ctx* ctx, int64_t total_particles, int force);
-// After the pushes of a step: every binned species' tile frame moves by its frame velocity, and the
-// velocity becomes the cell displacement that at least 3/4 of the species' particles made in the
-// push just done (else 0); the displacement counts are cleared.
-pic_status particles_frames_advance(pic_ctx* ctx, const pic_species32* sp, int n_species);
+// The same for every species of a step at once (tiles of at most 4096 cells: bin32_two_level); offsets
+// and chunks: one array per species, frames: ctx->frame or nullptr.  home: keys by the nearest node
+// instead of the cell (shape order 2).  The sorted particles are in the species arrays afterwards.
+pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_species, int64_t* const* offsets,
+                                uint32_t* const* chunks, const int* gate, const int* frames, bool home);
+// The start of a step of the tiled form, one launch.  advance: after the pushes of the step before,
+// every binned species' tile frame moves by its frame velocity, and the velocity becomes the
+// displacement that at least 3/4 of the species' particles made in that push (else 0).  decide:
+// *bin_gate = (particles whose new home left their tile in the last tiled push > 2 % of all) || force.
+// zero_j, zero_rho (or nullptr): arrays of 3 ncell and ncell floats to clear.
+pic_status particles_begin32(pic_ctx* ctx, const pic_species32* sp, int n_species, bool advance, bool decide, bool force,
+                             float* zero_j, float* zero_rho);
 // device flag: the last particles_bin32 call permuted the species (its sorted copy is in bin_tmp)
 inline const int* bin32_scatter_gate(const pic_ctx* ctx) { return ctx->bin_flags + 1; }
 // tiles of at most 4096 cells are binned in two levels (by tile, then by cell inside each tile in
 // shared memory), which always leaves the sorted particles in the species arrays (copy_back is
 // implied); larger tiles by one counting sort over every cell
 bool bin32_two_level(const pic_ctx* ctx);
-// kernel launches of one particles_bin32 call (for the stage launch counters)
-int bin32_launches(const pic_ctx* ctx, int64_t n, bool chunks, bool copy_back);
+// kernel launches of binning n_species species in a step (for the stage launch counters)
+int bin32_launches(const pic_ctx* ctx, const pic_species32* sp, int n_species);
 
 // center.cu -------------------------------------------------------------------
 pic_status center_to_nodal(pic_ctx* ctx, const double* const F[6], double* const out[6]);
