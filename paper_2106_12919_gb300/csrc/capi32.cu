@@ -245,6 +245,7 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
   const bool early_bin = tiled && n_species > 0;
   const int nbin = std::min(n_species, PIC_MAX_BINNED_SPECIES);
   const bool two_level = bin32_two_level(ctx), home = ctx->shape_order == 2 && two_level;
+  const bool linear = tiled && bin32_linear(ctx);
   if (early_bin) {
     PIC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
     PIC_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
@@ -255,7 +256,7 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
       StageScope t(ctx, STAGE_BIN, 1 + bin32_launches(ctx, sp, two_level ? nbin : 1));
       st = particles_begin32(ctx, sp, n_species, false, true, true, nullptr, nullptr);
       if (st == PIC_OK)
-        st = two_level ? particles_bin32_step(ctx, sp, nbin, ctx->sp_off, ctx->sp_chunk, ctx->bin_gate, ctx->frame, home)
+        st = two_level ? particles_bin32_step(ctx, sp, nbin, ctx->sp_off, ctx->sp_chunk, ctx->bin_gate, ctx->frame, home, linear)
                        : particles_bin32(ctx, &sp[0], ctx->sp_off[0], ctx->bin_gate, ctx->sp_chunk[0], false, ctx->frame);
     }
     ctx->stream = main_stream;
@@ -311,7 +312,7 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
       PIC_TRY32(particles_begin32(ctx, sp, n_species, s > 0, !first, force, jn, rho));
       if (first) PIC_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
       else if (two_level && nbin > 0)
-        PIC_TRY32(particles_bin32_step(ctx, sp, nbin, ctx->sp_off, ctx->sp_chunk, ctx->bin_gate, ctx->frame, home));
+        PIC_TRY32(particles_bin32_step(ctx, sp, nbin, ctx->sp_off, ctx->sp_chunk, ctx->bin_gate, ctx->frame, home, linear));
     } else {
       PIC_CUDA_TRY(ctx, cudaMemsetAsync(jn, 0, 3 * nc * sizeof(float), ctx->stream));
       PIC_CUDA_TRY(ctx, cudaMemsetAsync(rho, 0, nc * sizeof(float), ctx->stream));
@@ -330,7 +331,7 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
         StageScope t(ctx, STAGE_PUSH, sp[q].n > 0 ? (ctx->vg[2] != 0.0 ? 2 : 1) : 0);
         PIC_TRY32(particles_push32_tiled(ctx, En, Bn, &sp[q], Jnp, rho, ctx->sp_off[q], ctx->sp_chunk[q],
                                          two_level ? nullptr : bin32_scatter_gate(ctx),
-                                         ctx->frame + 8 * q, ctx->dhist + 10 * q));
+                                         ctx->frame + 8 * q, ctx->dhist + 10 * q, linear));
       } else {
         StageScope t(ctx, STAGE_PUSH, sp[q].n > 0 ? 1 : 0);
         PIC_TRY32(particles_push32(ctx, En, Bn, &sp[q], Jnp, rho));

@@ -518,12 +518,12 @@ __global__ void __launch_bounds__(256) push32_stag_kernel(Push32Args a) {
 // the tile plus two guard cells on each side (enough for a cubic shape and a move of
 // up to one cell), and the window is flushed once with global atomics.
 //
-// Shared-memory layout.  Binning orders the cells of a tile z fastest, then x, then y,
-// so at P particles per cell the 32 lanes of a warp (visiting every P-th particle)
-// hold 32 cells: the T2 = 8 z-cells of 4 consecutive x-planes at one y.  Both shared arrays
-// are component-planar with the plane stride padded to 8 (mod 32) words, so the
-// lanes' addresses for the same relative node fall in 32 distinct banks: every
-// gather load and every deposit atomic of such a warp is one conflict-free access.
+// Shared-memory layout.  Both shared arrays are component-planar with the plane stride padded to 8 or
+// 24 (mod 32) words, and binning orders a tile's particles so that the 32 lanes of a warp hold cells
+// whose addresses for the same relative node fall in 32 distinct banks: one conflict-free access for
+// every gather load and deposit atomic.  The step's binning deals the particles out by that bank
+// (class_order_kernel, `linear`); otherwise the cells come z fastest, then x, then y, and at P particles
+// per cell the lanes visit every P-th particle: the T2 = 8 z-cells of 4 consecutive x-planes at one y.
 struct TileArgs {
   const int64_t* off;     // [n_tiles + 1] particle ranges
   const uint32_t* chunk;  // [n_tiles + 1] exclusive prefix sum of chunks per tile
@@ -536,7 +536,9 @@ struct TileArgs {
   int W[3];               // deposit window edge = T + 5
   int wplane, wcomp;      // deposit window plane and component strides (words)
   int G[3];               // gather window edge = T + 3: nodes [T0 - 1, T0 + T + 2)
+  int grow;               // gather window row stride
   int gplane, gcomp;      // gather window plane and component strides (words)
+  int linear;             // lanes take consecutive particles
   int vec_flush;          // flush by aligned groups of 4 z nodes (16-byte vector reductions)
 };
 
@@ -627,7 +629,7 @@ __global__ void __launch_bounds__(kTileThreads, 1024 / kTileThreads) push32_tile
   win.plane = t.wplane;
   win.comp = t.wcomp;
   win.acc = reinterpret_cast<int*>(smem);
-  const int G1 = t.G[1], G2 = t.G[2], gplane = t.gplane, gcomp = t.gcomp;
+  const int G1 = t.G[1], G2 = t.G[2], grow = t.grow, gplane = t.gplane, gcomp = t.gcomp;
   // the staged fields are needed in phase 1 only and the deposit window in phase 2 only:
   // both live at the start of the dynamic shared memory
   // [3][G0][G1][G2] pairs (E_x, E_y), (E_z, B_x), (B_y, B_z), plane stride gplane: one 8-byte load
@@ -647,7 +649,7 @@ __global__ void __launch_bounds__(kTileThreads, 1024 / kTileThreads) push32_tile
     const int k = e % G2, r = e / G2;
     const int j = r % G1, i = r / G1;
     const int o = (((go0 + i) & a.mask[0]) * (int)a.Ny + ((go1 + j) & a.mask[1])) * (int)a.Nz + ((go2 + k) & a.mask[2]);
-    const int d = i * gplane + j * G2 + k;
+    const int d = i * gplane + j * grow + k;
 #pragma unroll
     for (int q = 0; q < 3; ++q) fld[q * gcomp + d] = make_float2(__ldg(a.F[2 * q] + o), __ldg(a.F[2 * q + 1] + o));
   }
@@ -655,7 +657,7 @@ __global__ void __launch_bounds__(kTileThreads, 1024 / kTileThreads) push32_tile
   constexpr int NS = P + 1;
   // visit every s-th particle (s ~ the tile's particles per cell) so that a warp's lanes hold
   // distinct cells; a chunk of a dense tile spans only cnt / s cells, and its lanes spread over them
-  const int s = max(1, ppc);
+  const int s = t.linear ? 1 : max(1, ppc);
   const int q = (cnt + s - 1) / s;
   unsigned nout = 0;
   // Phase 1: gather, Boris push and move of every particle of the chunk; the new state goes to
@@ -709,7 +711,7 @@ __global__ void __launch_bounds__(kTileThreads, 1024 / kTileThreads) push32_tile
 #pragma unroll
         for (int jj = 0; jj < NS; ++jj) {
           const float sxy = Sx[i] * Sy[jj];
-          const float2* row = fld + (gx + i) * gplane + (gy + jj) * G2 + gz;
+          const float2* row = fld + (gx + i) * gplane + (gy + jj) * grow + gz;
 #pragma unroll
           for (int k = 0; k < NS; ++k) {
             const float w = sxy * Sz[k];
@@ -947,6 +949,9 @@ size_t chunk_map_offset(const pic_ctx* ctx) {
   return (size_t)ctx->n_tiles + 1 + (size_t)((ctx->n_tiles + kScanBlock - 1) / kScanBlock) + 1;
 }
 
+// dynamic shared memory a tile may take (tiled_push_fits)
+constexpr int kMaxTileSmem = 160 * 1024;
+
 // smallest stride >= v that is 8 or 24 (mod 32) words: a warp's lanes (8 z cells x 4 x planes)
 // then fall on 32 distinct banks (z + 8 x or z + 24 x, mod 32)
 int pad_plane(int v) {
@@ -958,8 +963,9 @@ int pad_plane(int v) {
 // The window spans the tile, 2 nodes before it and 3 after it on every axis (the cubic block of a
 // particle one cell past the tile), except 2 after it along x when wx_after = 2 (see
 // launch_push32_tiled): a particle that moved past the tile's upper x face since its binning then
-// deposits through global memory.
-size_t tile_layout(const pic_ctx* ctx, TileArgs& t, int wx_after) {
+// deposits through global memory.  linear: the gather rows take the window's row stride, so that one
+// class of cells is one bank in both arrays (class_order_kernel).
+size_t tile_layout(const pic_ctx* ctx, TileArgs& t, int wx_after, bool linear) {
   t.cpt = 1;
   for (int d = 0; d < 3; ++d) {
     t.T[d] = ctx->tile[d];
@@ -970,12 +976,39 @@ size_t tile_layout(const pic_ctx* ctx, TileArgs& t, int wx_after) {
   }
   t.wplane = pad_plane(t.W[1] * t.W[2]);
   t.wcomp = t.W[0] * t.wplane;
-  t.gplane = pad_plane(t.G[1] * t.G[2]);
+  t.grow = linear ? t.W[2] : t.G[2];
+  t.gplane = pad_plane(t.G[1] * t.grow);
   t.gcomp = t.G[0] * t.gplane;
+  t.linear = linear ? 1 : 0;
   return std::max(4 * (size_t)t.wcomp, 6 * (size_t)t.gcomp) * sizeof(float);
 }
 
-pic_status launch_push32_tiled(pic_ctx* ctx, const Push32Args& a, const int64_t* off, const uint32_t* chunk) {
+// the layout of the context's tiles with the most CTAs per SM: the window one node shorter along x when
+// that lets more of them share one (e.g. 8 x 16 x 8 tiles: 3 -> 4 CTAs, the register limit)
+pic_status choose_layout(pic_ctx* ctx, bool linear, TileArgs& t, size_t& smem, int* ctas = nullptr) {
+  smem = tile_layout(ctx, t, 3, linear);
+  TileArgs t2 = t;
+  const size_t smem2 = tile_layout(ctx, t2, 2, linear);
+  const void* fn = ctx->shape_order == 1 ? (const void*)push32_tile_kernel<1, false>
+                   : ctx->shape_order == 2 ? (const void*)push32_tile_kernel<2, false>
+                                           : (const void*)push32_tile_kernel<3, false>;
+  const void* fx = ctx->shape_order == 1 ? (const void*)push32_tile_kernel<1, true>
+                   : ctx->shape_order == 2 ? (const void*)push32_tile_kernel<2, true>
+                                           : (const void*)push32_tile_kernel<3, true>;
+  PIC_CUDA_TRY(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTileSmem));
+  PIC_CUDA_TRY(ctx, cudaFuncSetAttribute(fx, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTileSmem));
+  int n3 = 0, n2 = 0;
+  PIC_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n3, fn, kTileThreads, smem));
+  PIC_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n2, fn, kTileThreads, smem2));
+  if (n2 > n3) {
+    t = t2;
+    smem = smem2;
+  }
+  if (ctas) *ctas = std::max(n2, n3);
+  return PIC_OK;
+}
+
+pic_status launch_push32_tiled(pic_ctx* ctx, const Push32Args& a, const int64_t* off, const uint32_t* chunk, bool linear) {
   if (a.n == 0) return PIC_OK;
   TileArgs t;
   t.off = off;
@@ -983,28 +1016,8 @@ pic_status launch_push32_tiled(pic_ctx* ctx, const Push32Args& a, const int64_t*
   t.chunk_tile = chunk + chunk_map_offset(ctx);
   t.n_tiles = ctx->n_tiles;
   t.outside = ctx->bin_outside;
-  // the window one node shorter along x when that lets more CTAs share an SM (e.g. 8 x 16 x 8
-  // tiles: 3 -> 4 CTAs, the register limit)
-  size_t smem = tile_layout(ctx, t, 3);
-  {
-    TileArgs t2 = t;
-    const size_t smem2 = tile_layout(ctx, t2, 2);
-    const void* fn = ctx->shape_order == 1 ? (const void*)push32_tile_kernel<1, false>
-                     : ctx->shape_order == 2 ? (const void*)push32_tile_kernel<2, false>
-                                             : (const void*)push32_tile_kernel<3, false>;
-    const void* fx = ctx->shape_order == 1 ? (const void*)push32_tile_kernel<1, true>
-                     : ctx->shape_order == 2 ? (const void*)push32_tile_kernel<2, true>
-                                             : (const void*)push32_tile_kernel<3, true>;
-    PIC_CUDA_TRY(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PIC_CUDA_TRY(ctx, cudaFuncSetAttribute(fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int n3 = 0, n2 = 0;
-    PIC_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n3, fn, kTileThreads, smem));
-    PIC_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n2, fn, kTileThreads, smem2));
-    if (n2 > n3) {
-      t = t2;
-      smem = smem2;
-    }
-  }
+  size_t smem = 0;
+  PIC_TRY(choose_layout(ctx, linear, t, smem));
   bool aligned = ctx->N[2] % 4 == 0;
   const float* dsts[4] = {a.J[0], a.J[1], a.J[2], a.rho};
   for (const float* d : dsts) aligned = aligned && (reinterpret_cast<uintptr_t>(d) % 16 == 0);
@@ -1379,6 +1392,20 @@ __global__ void tile_count_kernel(BinBatch b) {
   flag_unsorted(a, mine);
 }
 
+// Class of a cell of the tile: the bank of its window node, z + plane x + row y (mod 32).  The step's
+// binning orders a tile's particles by (number within the class, class): as long as every class has
+// particles left, any 32 consecutive ones have 32 classes, so the lanes of a warp, which take
+// consecutive particles, share no bank and no cell.  (Ordered by cell instead, with lanes visiting
+// every P-th particle, lanes of one cell or of aliasing cells met as soon as the counts per cell varied:
+// 3.1 wavefronts per atomic instruction and 2.7 per 8-byte load instead of 1 and 2.)
+struct ClassArgs {
+  int plane, row;  // window strides (mod 32)
+};
+__device__ __forceinline__ int class_of(const Key32Args& k, const ClassArgs& c, int key) {
+  const int z = key & k.tmask[2], x = (key >> k.lshift_z) & k.tmask[0], y = (key >> (k.lshift_z + k.lshift_x)) & k.tmask[1];
+  return (z + c.plane * x + c.row * y) & 31;
+}
+
 struct BinScan {
   const int* gate;
   int n_tiles;
@@ -1388,6 +1415,7 @@ struct BinScan {
   uint32_t* chunk[PIC_MAX_BINNED_SPECIES];   // chunk starts [n_tiles + 1] or null
   uint32_t* cmap[PIC_MAX_BINNED_SPECIES];    // tile of each chunk
   int* flags;                                // + 2 q: keys out of order (cleared after use), scatter gate
+  int always;                                // permute whatever the order
 };
 
 // inclusive sum over the CTA's 1024 threads of a pair; red: 32 pairs
@@ -1462,20 +1490,20 @@ __global__ void __launch_bounds__(1024) bin_scan_kernel(BinScan a) {
   if (threadIdx.x == 0) {
     off[a.n_tiles] = (int64_t)base.x;
     if (chunk) chunk[a.n_tiles] = base.y;
-    a.flags[2 * q + 1] = a.flags[2 * q] != 0 ? 1 : 0;
+    a.flags[2 * q + 1] = (a.always || a.flags[2 * q] != 0) ? 1 : 0;
     a.flags[2 * q] = 0;
   }
 }
 
 // after the multi-kernel scan (see particles_bin32): the offsets, scanned in place, become the cursors
-__global__ void scan_finish_kernel(uint32_t* counts, uint32_t* cursor, int64_t n, int* flags, const int* gate) {
+__global__ void scan_finish_kernel(uint32_t* counts, uint32_t* cursor, int64_t n, int* flags, int always, const int* gate) {
   if (gated_off(gate)) return;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
     cursor[t] = counts[t];
     counts[t] = 0u;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    flags[1] = flags[0] != 0 ? 1 : 0;
+    flags[1] = (always || flags[0] != 0) ? 1 : 0;
     flags[0] = 0;
   }
 }
@@ -1604,6 +1632,64 @@ __global__ void __launch_bounds__(kOrderThreads) cell_order_kernel(TileScatterAr
   }
 }
 
+// level 2 of the step's binning: scratch -> species arrays, each tile in class order (see ClassArgs).
+// Particle r of class c goes to place sum_c' min(n_c', r) + #{c' < c: n_c' > r}; which particle of a
+// class is its r-th is up to the shared-memory atomics.  Copies as cell_order_kernel.
+__global__ void __launch_bounds__(kOrderThreads) class_order_kernel(TileScatterArgs a, ClassArgs ca, const int64_t* tile_off,
+                                                                    int64_t n_tiles) {
+  if (gated_off(a.gate) || *a.sgate == 0) return;
+  a.k = load_frame(a.k);
+  __shared__ uint32_t n[32], next[32];
+  __shared__ uint16_t rank[kMaxOrder], order[kMaxOrder];
+  const auto place = [&](int c, uint32_t r) {
+    uint32_t q = 0;
+#pragma unroll
+    for (int d = 0; d < 32; ++d) q += min(n[d], r) + (d < c && n[d] > r ? 1u : 0u);
+    return q;
+  };
+  for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+    const int64_t b0 = tile_off[t], nt = tile_off[t + 1] - b0;
+    if (nt == 0) continue;  // uniform over the CTA
+    if (threadIdx.x < 32) n[threadIdx.x] = next[threadIdx.x] = 0u;
+    __syncthreads();
+    const bool listed = nt <= kMaxOrder;
+    for (int64_t i = threadIdx.x; i < nt; i += blockDim.x) {
+      const uint32_t r = atomicAdd(&n[class_of(a.k, ca, tmp_key(a, b0 + i))], 1u);
+      if (listed) rank[i] = (uint16_t)r;
+    }
+    __syncthreads();
+    if (listed) {
+      for (int i = threadIdx.x; i < (int)nt; i += blockDim.x)
+        order[place(class_of(a.k, ca, tmp_key(a, b0 + i)), rank[i])] = (uint16_t)i;
+      __syncthreads();
+      for (int i = threadIdx.x; i < (int)nt; i += blockDim.x) {
+        const int64_t j = b0 + order[i];
+        uint32_t v[8];
+#pragma unroll
+        for (int f = 0; f < 8; ++f) v[f] = a.tmp[f][j];
+        const unsigned long long id = a.id_spc ? a.id_tmp[j] : 0ull;
+#pragma unroll
+        for (int f = 0; f < 8; ++f) a.spc[f][b0 + i] = v[f];
+        if (a.id_spc) a.id_spc[b0 + i] = id;
+      }
+    } else {
+      for (int64_t i = threadIdx.x; i < nt; i += blockDim.x) {
+        const int64_t j = b0 + i;
+        uint32_t v[8];
+#pragma unroll
+        for (int f = 0; f < 8; ++f) v[f] = a.tmp[f][j];
+        const unsigned long long id = a.id_spc ? a.id_tmp[j] : 0ull;
+        const int c = class_of(a.k, ca, word_key(a.k, v));
+        const int64_t q = b0 + place(c, atomicAdd(&next[c], 1u));
+#pragma unroll
+        for (int f = 0; f < 8; ++f) a.spc[f][q] = v[f];
+        if (a.id_spc) a.id_spc[q] = id;
+      }
+    }
+    __syncthreads();  // the shared arrays are reused by the next tile
+  }
+}
+
 }  // namespace
 
 #ifndef PIC_BIN_LIMIT
@@ -1672,7 +1758,7 @@ int bin32_launches(const pic_ctx* ctx, const pic_species32* sp, int n_species) {
 
 bool tiled_push_fits(const pic_ctx* ctx) {
   TileArgs t;
-  return tile_layout(ctx, t, 3) <= 160 * 1024 && ctx->ncell < (int64_t(1) << 31);
+  return tile_layout(ctx, t, 3, false) <= (size_t)kMaxTileSmem && ctx->ncell < (int64_t(1) << 31);
 }
 
 size_t tile_chunk_words(const pic_ctx* ctx, int64_t n) {
@@ -1683,7 +1769,7 @@ size_t tile_chunk_words(const pic_ctx* ctx, int64_t n) {
 pic_status particles_push32_tiled(pic_ctx* ctx, const float* const En[3], const float* const Bn[3],
                                   const pic_species32* sp, float* const J[3], float* rho, const int64_t* offsets,
                                   const uint32_t* chunks, const int* sorted_gate, const int* frame,
-                                  unsigned long long* dhist) {
+                                  unsigned long long* dhist, bool linear) {
   Push32Args a = make_args32(ctx, sp);
   a.frame = frame;
   a.dhist = dhist;
@@ -1703,7 +1789,7 @@ pic_status particles_push32_tiled(pic_ctx* ctx, const float* const En[3], const 
     a.id_dst = reinterpret_cast<unsigned long long*>(sp->id);
     a.w_dst = sp->w;
   }
-  return launch_push32_tiled(ctx, a, offsets, chunks);
+  return launch_push32_tiled(ctx, a, offsets, chunks, linear);
 }
 
 pic_status particles_deposit_rho32(pic_ctx* ctx, const pic_species32* sp, float* rho) {
@@ -1784,8 +1870,16 @@ static pic_status bin32_scratch(pic_ctx* ctx, int nsp) {
   return PIC_OK;
 }
 
+bool bin32_linear(pic_ctx* ctx) {
+  TileArgs t;
+  size_t smem;
+  int n0 = 0, n1 = 0;
+  return bin32_two_level(ctx) && choose_layout(ctx, false, t, smem, &n0) == PIC_OK && tile_layout(ctx, t, 2, true) <= (size_t)kMaxTileSmem &&
+         tile_layout(ctx, t, 3, true) <= (size_t)kMaxTileSmem && choose_layout(ctx, true, t, smem, &n1) == PIC_OK && n1 >= n0;
+}
+
 pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_species, int64_t* const* offsets,
-                                uint32_t* const* chunks, const int* gate, const int* frames, bool home) {
+                                uint32_t* const* chunks, const int* gate, const int* frames, bool home, bool linear) {
   PIC_TRY(bin32_scratch(ctx, n_species));
   int64_t nmax = 1;
   for (int q = 0; q < n_species; ++q) nmax = std::max(nmax, sp[q].n);
@@ -1798,6 +1892,7 @@ pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_spe
   b.gate = sc.gate = gate;
   sc.n_tiles = (int)nt;
   sc.flags = flags;
+  sc.always = linear ? 1 : 0;
   for (int q = 0; q < n_species; ++q) {
     Key32Args& k = b.k[q];
     k = key_args(ctx, &sp[q], frames ? frames + 8 * q : nullptr, home);
@@ -1831,7 +1926,7 @@ pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_spe
       scan_add_kernel<<<blocks(nt), 256, 0, ctx->stream>>>(sc.counts[q], nt, bsum, 0, sc.off[q], nt, total, gate);
       PIC_LAUNCH_CHECK(ctx);
       if (chunks) PIC_TRY(build_chunks(ctx, sc.off[q], sc.chunk[q], gate));
-      scan_finish_kernel<<<blocks(nt), 256, 0, ctx->stream>>>(sc.counts[q], sc.cursor[q], nt, flags + 2 * q, gate);
+      scan_finish_kernel<<<blocks(nt), 256, 0, ctx->stream>>>(sc.counts[q], sc.cursor[q], nt, flags + 2 * q, sc.always, gate);
       PIC_LAUNCH_CHECK(ctx);
     }
   }
@@ -1852,7 +1947,14 @@ pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_spe
     s.cursor = sc.cursor[q];
     tile_scatter_kernel<<<blocks(sp[q].n), bs, 0, ctx->stream>>>(s);
     PIC_LAUNCH_CHECK(ctx);
-    cell_order_kernel<<<(unsigned)std::min<int64_t>(nt, 152 * 8), kOrderThreads, 0, ctx->stream>>>(s, sc.off[q], nt);
+    const unsigned ob = (unsigned)std::min<int64_t>(nt, 152 * 8);
+    if (linear) {
+      TileArgs t;
+      tile_layout(ctx, t, 3, true);
+      class_order_kernel<<<ob, kOrderThreads, 0, ctx->stream>>>(s, ClassArgs{t.wplane & 31, t.W[2] & 31}, sc.off[q], nt);
+    } else {
+      cell_order_kernel<<<ob, kOrderThreads, 0, ctx->stream>>>(s, sc.off[q], nt);
+    }
     PIC_LAUNCH_CHECK(ctx);
   }
   return PIC_OK;
@@ -1863,7 +1965,7 @@ pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offse
   const int64_t n = sp->n;
   if (bin32_two_level(ctx)) {
     PIC_TRY(particles_bin_capacity(ctx, 1));  // bin_counts
-    return particles_bin32_step(ctx, sp, 1, &offsets_out, chunks_out ? &chunks_out : nullptr, gate, frame, false);
+    return particles_bin32_step(ctx, sp, 1, &offsets_out, chunks_out ? &chunks_out : nullptr, gate, frame, false, false);
   }
   PIC_TRY(particles_bin_capacity(ctx, n > 0 ? n : 1));
   const int64_t ncell = ctx->ncell;

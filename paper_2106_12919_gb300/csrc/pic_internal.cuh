@@ -382,7 +382,7 @@ pic_status particles_push32_tiled(pic_ctx* ctx, const float* const En[3], const 
                                   const pic_species32* sp, float* const J[3], float* rho, const int64_t* offsets,
                                   const uint32_t* chunks,
                                   const int* sorted_gate = nullptr, const int* frame = nullptr,
-                                  unsigned long long* dhist = nullptr);
+                                  unsigned long long* dhist = nullptr, bool linear = false);
 // gate: device flag; the binning kernels do nothing while *gate == 0 (nullptr = always bin).
 // chunks_out (optional, tile_chunk_words entries): chunk starts for particles_push32_tiled.
 // copy_back = false leaves the sorted particles in ctx->bin_tmp (the species arrays untouched) for
@@ -395,9 +395,13 @@ pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offse
                            uint32_t* chunks_out = nullptr, bool copy_back = true, const int* frame = nullptr);
 // The same for every species of a step at once (tiles of at most 4096 cells: bin32_two_level); offsets
 // and chunks: one array per species, frames: ctx->frame or nullptr.  home: keys by the nearest node
-// instead of the cell (shape order 2).  The sorted particles are in the species arrays afterwards.
+// instead of the cell (shape order 2).  linear: the order inside a tile for a push with linear set
+// (class_order_kernel) instead of by cell.  The sorted particles are in the species arrays afterwards.
 pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_species, int64_t* const* offsets,
-                                uint32_t* const* chunks, const int* gate, const int* frames, bool home);
+                                uint32_t* const* chunks, const int* gate, const int* frames, bool home, bool linear);
+// whether the step's binning and push use that order: its shared-memory layout (longer gather rows) must
+// not cost CTAs per SM (8 x 16 x 8 tiles: 3 instead of 4, and they keep the order by cell)
+bool bin32_linear(pic_ctx* ctx);
 // The start of a step of the tiled form, one launch.  advance: after the pushes of the step before,
 // every binned species' tile frame moves by its frame velocity, and the velocity becomes the
 // displacement that at least 3/4 of the species' particles made in that push (else 0).  decide:
