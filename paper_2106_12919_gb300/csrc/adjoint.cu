@@ -260,23 +260,20 @@ bool nonnull(P const* a, int n) {
     if (s_ != PIC_OK) return s_;   \
   } while (0)
 
-const int kKindEB[6] = {0, 1, 2, 3, 4, 5};
-
-// Yee real arrays -> paper-convention spectra in ctx->EBh (through G)
-pic_status to_paper(pic_ctx* ctx, const double* const* F6) {
+// Yee real arrays -> paper-convention spectra in ctx->EBh; nodal: G = the DFT of the nodal fields / Ncell
+pic_status to_paper(pic_ctx* ctx, const double* const* F6, bool nodal) {
   CRPtr6 in;
-  CPtr6 g, eb;
+  CPtr6 g;
   for (int c = 0; c < 6; ++c) {
     in.p[c] = F6[c];
     g.p[c] = ctx->G + c * ctx->nmode;
-    eb.p[c] = ctx->EBh + c * ctx->nmode;
   }
   {
     StageScope t(ctx, STAGE_FFT, 3);
     ADJ_TRY(fft_r2c<double>(ctx, in, g, 6));
   }
   StageScope t(ctx, STAGE_OTHER, 1);
-  return psatd_phase(ctx, g, eb, kKindEB, 6, -1, 1.0);
+  return psatd_load<double2>(ctx, ctx->G, ctx->EBh, nodal);
 }
 
 }  // namespace
@@ -320,11 +317,7 @@ extern "C" pic_status pic_adjoint_step(pic_ctx* ctx, const double* const E[3], c
   double* fb = ctx->adj_work + 2 * nc;    // [6] nodal force adjoints
   // 1. nodal E, B at t^n (forward recompute)
   const double* F6[6] = {E[0], E[1], E[2], B[0], B[1], B[2]};
-  ADJ_TRY(to_paper(ctx, F6));
-  {
-    StageScope t(ctx, STAGE_OTHER, 1);
-    ADJ_TRY(psatd_to_nodal(ctx, ctx->EBh, 1.0 / (double)nc));
-  }
+  ADJ_TRY(to_paper(ctx, F6, true));
   {
     CPtr6 g;
     RPtr6 o;
@@ -337,7 +330,7 @@ extern "C" pic_status pic_adjoint_step(pic_ctx* ctx, const double* const E[3], c
   }
   // 2. transpose of the update on the incoming field adjoints
   const double* Fb6[6] = {Ebar[0], Ebar[1], Ebar[2], Bbar[0], Bbar[1], Bbar[2]};
-  ADJ_TRY(to_paper(ctx, Fb6));
+  ADJ_TRY(to_paper(ctx, Fb6, false));
   {
     StageScope t(ctx, STAGE_UPDATE, 1);
     ADJ_TRY(psatd_adjoint_update(ctx, ctx->EBh, ctx->G));
@@ -420,19 +413,16 @@ extern "C" pic_status pic_adjoint_step(pic_ctx* ctx, const double* const E[3], c
     ADJ_TRY(psatd_add_zeta(ctx, ctx->EBh, ctx->G));
   }
   {
-    CPtr6 s6, g;
+    CPtr6 g;
     RPtr6 o;
-    for (int c = 0; c < 6; ++c) {
-      s6.p[c] = ctx->EBh + c * nm;
-      g.p[c] = ctx->G + c * nm;
-    }
+    for (int c = 0; c < 6; ++c) g.p[c] = ctx->G + c * nm;
     for (int c = 0; c < 3; ++c) {
       o.p[c] = Ebar[c];
       o.p[3 + c] = Bbar[c];
     }
     {
       StageScope t(ctx, STAGE_OTHER, 1);
-      ADJ_TRY(psatd_phase(ctx, s6, g, kKindEB, 6, +1, 1.0 / (double)nc));
+      ADJ_TRY(psatd_store<double2>(ctx, ctx->EBh, ctx->G));
     }
     StageScope t(ctx, STAGE_FFT, 3);
     ADJ_TRY(fft_c2r<double>(ctx, g, o, 6));

@@ -62,27 +62,40 @@ bool all_nonnull(P const* a, int n) {
   return true;
 }
 
-const int kKindEB[6] = {0, 1, 2, 3, 4, 5};
 const int kKindJ[3] = {6, 7, 8};
 
-// Yee E, B (real) -> ctx->EBh (paper-convention spectra), via G as scratch.
-pic_status load_fields(pic_ctx* ctx, const double* const E[3], const double* const B[3]) {
+// Yee E, B (real) -> ctx->EBh (paper-convention spectra), via G as scratch; nodal: G = the DFT of the
+// nodal fields / Ncell.
+pic_status load_fields(pic_ctx* ctx, const double* const E[3], const double* const B[3], bool nodal) {
   CRPtr6 in;
-  CPtr6 g, eb;
+  CPtr6 g;
   for (int c = 0; c < 3; ++c) {
     in.p[c] = E[c];
     in.p[3 + c] = B[c];
   }
-  for (int c = 0; c < 6; ++c) {
-    g.p[c] = ctx->G + c * ctx->nmode;
-    eb.p[c] = ctx->EBh + c * ctx->nmode;
-  }
+  for (int c = 0; c < 6; ++c) g.p[c] = ctx->G + c * ctx->nmode;
   {
     StageScope t(ctx, STAGE_FFT, 3);
     PIC_TRY(fft_r2c(ctx, in, g, 6));
   }
   StageScope t(ctx, STAGE_OTHER, 1);
-  return psatd_phase(ctx, g, eb, kKindEB, 6, -1, 1.0);
+  return psatd_load<double2>(ctx, ctx->G, ctx->EBh, nodal);
+}
+
+// ctx->EBh -> Yee E, B, through G.
+pic_status store_fields(pic_ctx* ctx, double* const E[3], double* const B[3]) {
+  CPtr6 g;
+  RPtr6 o;
+  for (int c = 0; c < 6; ++c) {
+    g.p[c] = ctx->G + c * ctx->nmode;
+    o.p[c] = c < 3 ? E[c] : B[c - 3];
+  }
+  {
+    StageScope t(ctx, STAGE_OTHER, 1);
+    PIC_TRY(psatd_store<double2>(ctx, ctx->EBh, ctx->G));
+  }
+  StageScope t(ctx, STAGE_FFT, 3);
+  return fft_c2r(ctx, g, o, 6);
 }
 
 // spectra (paper convention) -> Yee real arrays, through G.
@@ -391,7 +404,7 @@ pic_status pic_maxwell_step(pic_ctx* ctx, double* const E[3], double* const B[3]
     return pic_set_error(ctx, PIC_ERR_ARG, "averaged variant needs Eavg, Bavg");
   const double* cE[3] = {E[0], E[1], E[2]};
   const double* cB[3] = {B[0], B[1], B[2]};
-  PIC_TRY(load_fields(ctx, cE, cB));
+  PIC_TRY(load_fields(ctx, cE, cB, false));
   // J (Yee) -> Jh paper convention; rho^n, rho^{n+1} -> rhoh
   CRPtr6 in;
   CPtr6 g, jh;
@@ -420,8 +433,7 @@ pic_status pic_maxwell_step(pic_ctx* ctx, double* const E[3], double* const B[3]
     for (int c = 0; c < 6; ++c) gg.p[c] = ctx->G + c * ctx->nmode;
     PIC_TRY(fft_c2r(ctx, gg, o, 6));
   }
-  double* outs[6] = {E[0], E[1], E[2], B[0], B[1], B[2]};
-  return store_yee(ctx, ctx->EBh, kKindEB, 6, outs);
+  return store_fields(ctx, E, B);
 }
 
 pic_status pic_coefficient(pic_ctx* ctx, const char* name, double* out) {
@@ -483,7 +495,8 @@ pic_status pic_step(pic_ctx* ctx, double* const E[3], double* const B[3], double
   // entry: spectral E^n, B^n, rho^n; nodal gather fields
   const double* cE[3] = {E[0], E[1], E[2]};
   const double* cB[3] = {B[0], B[1], B[2]};
-  PIC_TRY(load_fields(ctx, cE, cB));
+  const bool stag = ctx->cycle == PIC_CYCLE_STAGGERED;
+  PIC_TRY(load_fields(ctx, cE, cB, !stag));
   int cur = 0;
   {
     CRPtr6 rin;
@@ -493,7 +506,6 @@ pic_status pic_step(pic_ctx* ctx, double* const E[3], double* const B[3], double
     StageScope t(ctx, STAGE_FFT, 3);
     PIC_TRY(fft_r2c(ctx, rin, rout, 1));
   }
-  const bool stag = ctx->cycle == PIC_CYCLE_STAGGERED;
   if (stag) {
     // staggered comparison cycle: the first gather reads the caller's Yee E, B as they are
     const double* src[6] = {E[0], E[1], E[2], B[0], B[1], B[2]};
@@ -501,10 +513,6 @@ pic_status pic_step(pic_ctx* ctx, double* const E[3], double* const B[3], double
       PIC_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->nodal + c * nc, src[c], nc * sizeof(double), cudaMemcpyDeviceToDevice,
                                         ctx->stream));
   } else {
-    {
-      StageScope t(ctx, STAGE_OTHER, 1);
-      PIC_TRY(psatd_to_nodal(ctx, ctx->EBh, 1.0 / (double)nc));
-    }
     PIC_TRY(g_to_nodal(ctx));
   }
   const double* En[3] = {ctx->nodal, ctx->nodal + nc, ctx->nodal + 2 * nc};
@@ -553,8 +561,7 @@ pic_status pic_step(pic_ctx* ctx, double* const E[3], double* const B[3], double
     ++ctx->steps_done;
   }
   // exit: Yee E, B and J
-  double* outs[6] = {E[0], E[1], E[2], B[0], B[1], B[2]};
-  PIC_TRY(store_yee(ctx, ctx->EBh, kKindEB, 6, outs));
+  PIC_TRY(store_fields(ctx, E, B));
   if (!J) return PIC_OK;
   double* jouts[3] = {J[0], J[1], J[2]};
   return store_yee(ctx, ctx->Jh, kKindJ, 3, jouts);

@@ -42,7 +42,6 @@ pic_status check_species32(pic_ctx* ctx, const pic_species32* sp, int n_species)
   return PIC_OK;
 }
 
-const int kKindEB[6] = {0, 1, 2, 3, 4, 5};
 const int kKindJ[3] = {6, 7, 8};
 
 inline float2* f2(double2* p) { return reinterpret_cast<float2*>(p); }
@@ -55,23 +54,36 @@ float2* rhoh(pic_ctx* ctx, int k) { return f2(ctx->rhoh[0]) + k * ctx->nmode; }
 float* nodal(pic_ctx* ctx) { return f1(ctx->nodal); }
 float* Jn(pic_ctx* ctx) { return f1(ctx->Jn); }
 
-pic_status load_fields32(pic_ctx* ctx, const float* const E[3], const float* const B[3]) {
+// (nodal: G = the DFT of the nodal fields / Ncell)
+pic_status load_fields32(pic_ctx* ctx, const float* const E[3], const float* const B[3], bool nodal) {
   CRP6<float> in;
-  CP6<float2> g, eb;
+  CP6<float2> g;
   for (int c = 0; c < 3; ++c) {
     in.p[c] = E[c];
     in.p[3 + c] = B[c];
   }
-  for (int c = 0; c < 6; ++c) {
-    g.p[c] = Gs(ctx) + c * ctx->nmode;
-    eb.p[c] = EBh(ctx) + c * ctx->nmode;
-  }
+  for (int c = 0; c < 6; ++c) g.p[c] = Gs(ctx) + c * ctx->nmode;
   {
     StageScope t(ctx, STAGE_FFT, 3);
     PIC_TRY32(fft_r2c<float>(ctx, in, g, 6));
   }
   StageScope t(ctx, STAGE_OTHER, 1);
-  return psatd_phase32(ctx, g, eb, kKindEB, 6, -1, 1.0);
+  return psatd_load<float2>(ctx, Gs(ctx), EBh(ctx), nodal);
+}
+
+pic_status store_fields32(pic_ctx* ctx, float* const E[3], float* const B[3]) {
+  CP6<float2> g;
+  RP6<float> o;
+  for (int c = 0; c < 6; ++c) {
+    g.p[c] = Gs(ctx) + c * ctx->nmode;
+    o.p[c] = c < 3 ? E[c] : B[c - 3];
+  }
+  {
+    StageScope t(ctx, STAGE_OTHER, 1);
+    PIC_TRY32(psatd_store<float2>(ctx, EBh(ctx), Gs(ctx)));
+  }
+  StageScope t(ctx, STAGE_FFT, 3);
+  return fft_c2r<float>(ctx, g, o, 6);
 }
 
 pic_status store_yee32(pic_ctx* ctx, const float2* src, const int* kinds, int ncomp, float* const* out) {
@@ -265,7 +277,7 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
   }
   int cur = 0;
   if (!fd) {
-    PIC_TRY32(load_fields32(ctx, cE, cB));
+    PIC_TRY32(load_fields32(ctx, cE, cB, !stag));
     CRP6<float> rin;
     CP6<float2> rout;
     rin.p[0] = rho;
@@ -284,10 +296,6 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
       PIC_CUDA_TRY(ctx, cudaMemcpyAsync(nodal(ctx) + c * nc, src[c], nc * sizeof(float), cudaMemcpyDeviceToDevice,
                                         ctx->stream));
   } else {
-    {
-      StageScope t(ctx, STAGE_OTHER, 1);
-      PIC_TRY32(psatd_to_nodal32(ctx, EBh(ctx), Gs(ctx), 1.0 / (double)nc));
-    }
     PIC_TRY32(g_to_nodal32(ctx));
   }
   float* nd = nodal(ctx);
@@ -391,8 +399,7 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
     ++ctx->steps_done;
   }
   if (fd) return PIC_OK;
-  float* outs[6] = {E[0], E[1], E[2], B[0], B[1], B[2]};
-  PIC_TRY32(store_yee32(ctx, EBh(ctx), kKindEB, 6, outs));
+  PIC_TRY32(store_fields32(ctx, E, B));
   if (!J) return PIC_OK;
   float* jouts[3] = {J[0], J[1], J[2]};
   return store_yee32(ctx, Jh(ctx), kKindJ, 3, jouts);

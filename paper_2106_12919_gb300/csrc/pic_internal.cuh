@@ -275,14 +275,17 @@ pic_status psatd_update_ex(pic_ctx* ctx, const double2* rn, const double2* rp, i
 // comp_kind[c]: 0..5 = Ex..Bz, 6..8 = Jx..Jz, 9 = rho.
 pic_status psatd_phase(pic_ctx* ctx, CPtr6 in, CPtr6 out, const int* comp_kind, int ncomp, int sign,
                        double scale);
-// G[c] = Z_c * src[c] * scale, src = the six E,B spectra given (paper convention) -> nodal DFT.
-pic_status psatd_to_nodal(pic_ctx* ctx, const double2* EB6, double scale);
+// Six field spectra, [6][nmode] each.  load: G holds the DFT of the Yee fields; EB = its paper convention,
+// and with nodal G = the DFT of the nodal fields / Ncell.  store: G = the DFT of the Yee fields of EB / Ncell.
+template <class C>
+pic_status psatd_load(pic_ctx* ctx, C* G, C* EB, bool nodal);
+template <class C>
+pic_status psatd_store(pic_ctx* ctx, const C* EB, C* G);
 // FP32-form counterparts (FP32 spectra, FP64 tables rounded at use).
 pic_status psatd_update32(pic_ctx* ctx, float2* EB, float2* J, const float2* rn, const float2* rp, float2* G,
                           int g_mode, int j_yee, int write_j, int smooth);
 pic_status psatd_phase32(pic_ctx* ctx, CP6<float2> in, CP6<float2> out, const int* comp_kind, int ncomp, int sign,
                          double scale);
-pic_status psatd_to_nodal32(pic_ctx* ctx, const float2* EB6, float2* G, double scale);
 // Reverse mode (adjoint.cu): conjugate-transposed update on the adjoint spectra in EB (paper
 // convention, in place); G[0..2] = zeta * Jbar / Ncell (nodal DFT), G[3] = rhobar^n / Ncell,
 // G[4] = rhobar^{n+1} / Ncell.
