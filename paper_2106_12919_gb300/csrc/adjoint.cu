@@ -260,8 +260,8 @@ bool nonnull(P const* a, int n) {
     if (s_ != PIC_OK) return s_;   \
   } while (0)
 
-// Yee real arrays -> paper-convention spectra in ctx->EBh; nodal: G = the DFT of the nodal fields / Ncell
-pic_status to_paper(pic_ctx* ctx, const double* const* F6, bool nodal) {
+// Yee real arrays -> paper-convention spectra in ctx->EBh (through G)
+pic_status to_paper(pic_ctx* ctx, const double* const* F6) {
   CRPtr6 in;
   CPtr6 g;
   for (int c = 0; c < 6; ++c) {
@@ -273,7 +273,7 @@ pic_status to_paper(pic_ctx* ctx, const double* const* F6, bool nodal) {
     ADJ_TRY(fft_r2c<double>(ctx, in, g, 6));
   }
   StageScope t(ctx, STAGE_OTHER, 1);
-  return psatd_load<double2>(ctx, ctx->G, ctx->EBh, nodal);
+  return psatd_load<double2>(ctx, ctx->G, ctx->EBh);
 }
 
 }  // namespace
@@ -315,22 +315,17 @@ extern "C" pic_status pic_adjoint_step(pic_ctx* ctx, const double* const E[3], c
   double* rbn = ctx->adj_work;            // rhobar^n
   double* rbp = ctx->adj_work + nc;       // rhobar^{n+1} from the update
   double* fb = ctx->adj_work + 2 * nc;    // [6] nodal force adjoints
-  // 1. nodal E, B at t^n (forward recompute)
+  // 1. nodal E, B at t^n (forward recompute): centered in real space (work array: Jn, free until step 2)
   const double* F6[6] = {E[0], E[1], E[2], B[0], B[1], B[2]};
-  ADJ_TRY(to_paper(ctx, F6, true));
   {
-    CPtr6 g;
-    RPtr6 o;
-    for (int c = 0; c < 6; ++c) {
-      g.p[c] = ctx->G + c * nm;
-      o.p[c] = ctx->nodal + c * nc;
-    }
-    StageScope t(ctx, STAGE_FFT, 3);
-    ADJ_TRY(fft_c2r<double>(ctx, g, o, 6));
+    double* nodal6[6];
+    for (int c = 0; c < 6; ++c) nodal6[c] = ctx->nodal + c * nc;
+    StageScope t(ctx, STAGE_OTHER, center_launches(ctx, true));
+    ADJ_TRY(center_to_nodal(ctx, F6, nodal6));
   }
   // 2. transpose of the update on the incoming field adjoints
   const double* Fb6[6] = {Ebar[0], Ebar[1], Ebar[2], Bbar[0], Bbar[1], Bbar[2]};
-  ADJ_TRY(to_paper(ctx, Fb6, false));
+  ADJ_TRY(to_paper(ctx, Fb6));
   {
     StageScope t(ctx, STAGE_UPDATE, 1);
     ADJ_TRY(psatd_adjoint_update(ctx, ctx->EBh, ctx->G));

@@ -64,9 +64,8 @@ bool all_nonnull(P const* a, int n) {
 
 const int kKindJ[3] = {6, 7, 8};
 
-// Yee E, B (real) -> ctx->EBh (paper-convention spectra), via G as scratch; nodal: G = the DFT of the
-// nodal fields / Ncell.
-pic_status load_fields(pic_ctx* ctx, const double* const E[3], const double* const B[3], bool nodal) {
+// Yee E, B (real) -> ctx->EBh (paper-convention spectra), via G as scratch.
+pic_status load_fields(pic_ctx* ctx, const double* const E[3], const double* const B[3]) {
   CRPtr6 in;
   CPtr6 g;
   for (int c = 0; c < 3; ++c) {
@@ -79,7 +78,7 @@ pic_status load_fields(pic_ctx* ctx, const double* const E[3], const double* con
     PIC_TRY(fft_r2c(ctx, in, g, 6));
   }
   StageScope t(ctx, STAGE_OTHER, 1);
-  return psatd_load<double2>(ctx, ctx->G, ctx->EBh, nodal);
+  return psatd_load<double2>(ctx, ctx->G, ctx->EBh);
 }
 
 // ctx->EBh -> Yee E, B, through G.
@@ -404,7 +403,7 @@ pic_status pic_maxwell_step(pic_ctx* ctx, double* const E[3], double* const B[3]
     return pic_set_error(ctx, PIC_ERR_ARG, "averaged variant needs Eavg, Bavg");
   const double* cE[3] = {E[0], E[1], E[2]};
   const double* cB[3] = {B[0], B[1], B[2]};
-  PIC_TRY(load_fields(ctx, cE, cB, false));
+  PIC_TRY(load_fields(ctx, cE, cB));
   // J (Yee) -> Jh paper convention; rho^n, rho^{n+1} -> rhoh
   CRPtr6 in;
   CPtr6 g, jh;
@@ -496,7 +495,7 @@ pic_status pic_step(pic_ctx* ctx, double* const E[3], double* const B[3], double
   const double* cE[3] = {E[0], E[1], E[2]};
   const double* cB[3] = {B[0], B[1], B[2]};
   const bool stag = ctx->cycle == PIC_CYCLE_STAGGERED;
-  PIC_TRY(load_fields(ctx, cE, cB, !stag));
+  PIC_TRY(load_fields(ctx, cE, cB));
   int cur = 0;
   {
     CRPtr6 rin;
@@ -506,15 +505,22 @@ pic_status pic_step(pic_ctx* ctx, double* const E[3], double* const B[3], double
     StageScope t(ctx, STAGE_FFT, 3);
     PIC_TRY(fft_r2c(ctx, rin, rout, 1));
   }
-  if (stag) {
-    // staggered comparison cycle: the first gather reads the caller's Yee E, B as they are
-    const double* src[6] = {E[0], E[1], E[2], B[0], B[1], B[2]};
-    for (int c = 0; c < 6; ++c)
-      PIC_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->nodal + c * nc, src[c], nc * sizeof(double), cudaMemcpyDeviceToDevice,
-                                        ctx->stream));
+  // The first gather's fields: the caller's, centered to the nodes in real space (six inverse transforms
+  // less than from their spectra).  Staggered and nodal comparison cycles: as they are.
+  const double* src[6] = {E[0], E[1], E[2], B[0], B[1], B[2]};
+  double* nodal6[6];
+  for (int c = 0; c < 6; ++c) nodal6[c] = ctx->nodal + c * nc;
+  const bool centered = ctx->cycle == PIC_CYCLE_HYBRID;
+  if (centered) {
+    StageScope t(ctx, STAGE_OTHER, center_launches(ctx, true));
+    PIC_TRY(center_to_nodal(ctx, src, nodal6));
   } else {
-    PIC_TRY(g_to_nodal(ctx));
+    for (int c = 0; c < 6; ++c)
+      PIC_CUDA_TRY(ctx, cudaMemcpyAsync(nodal6[c], src[c], nc * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
   }
+  // The J of the last step goes back from its nodal (staggered cycle: Yee) deposit in real space as
+  // well, unless the bilinear filter, applied in Fourier space, is on.
+  const bool j_spectral = J && ctx->filter_passes > 0;
   const double* En[3] = {ctx->nodal, ctx->nodal + nc, ctx->nodal + 2 * nc};
   const double* Bn[3] = {ctx->nodal + 3 * nc, ctx->nodal + 4 * nc, ctx->nodal + 5 * nc};
   double* Jn[3] = {ctx->Jn, ctx->Jn + nc, ctx->Jn + 2 * nc};
@@ -554,7 +560,7 @@ pic_status pic_step(pic_ctx* ctx, double* const E[3], double* const B[3], double
       // hybrid: J nodal (centered in the update), G = nodal E, B; staggered: J and G on the Yee grid
       StageScope t(ctx, STAGE_UPDATE, 1);
       PIC_TRY(psatd_update_ex(ctx, ctx->rhoh[cur], ctx->rhoh[1 - cur], stag ? 1 : 0, stag ? 1 : 0,
-                              (last && J) ? 1 : 0, 1));
+                              (last && j_spectral) ? 1 : 0, 1));
     }
     cur = 1 - cur;
     if (!last) PIC_TRY(g_to_nodal(ctx));
@@ -563,6 +569,16 @@ pic_status pic_step(pic_ctx* ctx, double* const E[3], double* const B[3], double
   // exit: Yee E, B and J
   PIC_TRY(store_fields(ctx, E, B));
   if (!J) return PIC_OK;
+  if (!j_spectral && centered) {
+    StageScope t(ctx, STAGE_OTHER, center_launches(ctx, false));
+    const double* cJ[3] = {Jn[0], Jn[1], Jn[2]};
+    return center_to_yee(ctx, cJ, J);
+  }
+  if (!j_spectral) {
+    for (int c = 0; c < 3; ++c)
+      PIC_CUDA_TRY(ctx, cudaMemcpyAsync(J[c], Jn[c], nc * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
+    return PIC_OK;
+  }
   double* jouts[3] = {J[0], J[1], J[2]};
   return store_yee(ctx, ctx->Jh, kKindJ, 3, jouts);
 }

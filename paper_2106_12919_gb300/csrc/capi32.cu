@@ -54,8 +54,7 @@ float2* rhoh(pic_ctx* ctx, int k) { return f2(ctx->rhoh[0]) + k * ctx->nmode; }
 float* nodal(pic_ctx* ctx) { return f1(ctx->nodal); }
 float* Jn(pic_ctx* ctx) { return f1(ctx->Jn); }
 
-// (nodal: G = the DFT of the nodal fields / Ncell)
-pic_status load_fields32(pic_ctx* ctx, const float* const E[3], const float* const B[3], bool nodal) {
+pic_status load_fields32(pic_ctx* ctx, const float* const E[3], const float* const B[3]) {
   CRP6<float> in;
   CP6<float2> g;
   for (int c = 0; c < 3; ++c) {
@@ -68,7 +67,7 @@ pic_status load_fields32(pic_ctx* ctx, const float* const E[3], const float* con
     PIC_TRY32(fft_r2c<float>(ctx, in, g, 6));
   }
   StageScope t(ctx, STAGE_OTHER, 1);
-  return psatd_load<float2>(ctx, Gs(ctx), EBh(ctx), nodal);
+  return psatd_load<float2>(ctx, Gs(ctx), EBh(ctx));
 }
 
 pic_status store_fields32(pic_ctx* ctx, float* const E[3], float* const B[3]) {
@@ -277,7 +276,7 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
   }
   int cur = 0;
   if (!fd) {
-    PIC_TRY32(load_fields32(ctx, cE, cB, !stag));
+    PIC_TRY32(load_fields32(ctx, cE, cB));
     CRP6<float> rin;
     CP6<float2> rout;
     rin.p[0] = rho;
@@ -285,19 +284,20 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
     StageScope t(ctx, STAGE_FFT, 3);
     PIC_TRY32(fft_r2c<float>(ctx, rin, rout, 1));
   }
-  if (fd) {
-    // E^n, B^n -> nodes in real space (work arrays: the nodal J buffer, free until the deposit)
-    StageScope t(ctx, STAGE_OTHER, 9);
-    PIC_TRY32(center_to_nodal_t<float>(ctx, yee, nodal6, Jn(ctx), Jn(ctx) + nc));
-  } else if (stag) {
-    // staggered comparison cycle: the first gather reads the caller's Yee E, B as they are
-    const float* src[6] = {E[0], E[1], E[2], B[0], B[1], B[2]};
-    for (int c = 0; c < 6; ++c)
-      PIC_CUDA_TRY(ctx, cudaMemcpyAsync(nodal(ctx) + c * nc, src[c], nc * sizeof(float), cudaMemcpyDeviceToDevice,
-                                        ctx->stream));
+  // The first gather's fields: the caller's, centered to the nodes in real space (for the spectral cycles
+  // six inverse transforms less than from their spectra; work array: the nodal J buffer, free until the
+  // deposit).  Staggered and nodal comparison cycles: as they are.
+  const bool centered = fd || ctx->cycle == PIC_CYCLE_HYBRID;
+  if (centered) {
+    StageScope t(ctx, STAGE_OTHER, center_launches(ctx, true));
+    PIC_TRY32(center_to_nodal_t<float>(ctx, yee, nodal6, Jn(ctx)));
   } else {
-    PIC_TRY32(g_to_nodal32(ctx));
+    for (int c = 0; c < 6; ++c)
+      PIC_CUDA_TRY(ctx, cudaMemcpyAsync(nodal6[c], yee[c], nc * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
   }
+  // The J of the last step goes back from its nodal (staggered cycle: Yee) deposit in real space as
+  // well, unless the bilinear filter, applied in Fourier space, is on.
+  const bool j_spectral = J && ctx->filter_passes > 0;
   float* nd = nodal(ctx);
   const float* En[3] = {nd, nd + nc, nd + 2 * nc};
   const float* Bn[3] = {nd + 3 * nc, nd + 4 * nc, nd + 5 * nc};
@@ -354,17 +354,17 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
       // J^{n+1/2}: optional smoothing, nodes -> Yee (work arrays: the nodal E, B, free after the
       // push), leapfrog of E, B, then E^{n+1}, B^{n+1} -> nodes for the next gather
       {
-        StageScope t(ctx, STAGE_OTHER, 3 + 9 * ctx->filter_passes);
+        StageScope t(ctx, STAGE_OTHER, center_launches(ctx, false) + 9 * ctx->filter_passes);
         for (int c = 0; c < 3 && ctx->filter_passes > 0; ++c)
           PIC_TRY32(bilinear_filter_t<float>(ctx, Jnp[c], ctx->filter_passes, nodal(ctx), nodal(ctx) + nc));
         const float* cJn[3] = {Jnp[0], Jnp[1], Jnp[2]};
-        PIC_TRY32(center_to_yee_t<float>(ctx, cJn, Jy, nodal(ctx), nodal(ctx) + nc));
+        PIC_TRY32(center_to_yee_t<float>(ctx, cJn, Jy));
       }
       const float* cJ[3] = {Jy[0], Jy[1], Jy[2]};
       PIC_TRY32(fdtd_update32(ctx, E, B, cJ));
       if (!last) {
-        StageScope t(ctx, STAGE_OTHER, 9);
-        PIC_TRY32(center_to_nodal_t<float>(ctx, yee, nodal6, Jn(ctx), Jn(ctx) + nc));
+        StageScope t(ctx, STAGE_OTHER, center_launches(ctx, true));
+        PIC_TRY32(center_to_nodal_t<float>(ctx, yee, nodal6, Jn(ctx)));
       }
       ++ctx->steps_done;
       continue;
@@ -392,7 +392,7 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
       // hybrid: J nodal (centered in the update), G = nodal E, B; staggered: J and G on the Yee grid
       StageScope t(ctx, STAGE_UPDATE, 1);
       PIC_TRY32(psatd_update32(ctx, EBh(ctx), Jh(ctx), rhoh(ctx, cur), rhoh(ctx, 1 - cur), Gs(ctx), stag ? 1 : 0,
-                               stag ? 1 : 0, (last && J) ? 1 : 0, 1));
+                               stag ? 1 : 0, (last && j_spectral) ? 1 : 0, 1));
     }
     cur = 1 - cur;
     if (!last) PIC_TRY32(g_to_nodal32(ctx));
@@ -401,6 +401,16 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
   if (fd) return PIC_OK;
   PIC_TRY32(store_fields32(ctx, E, B));
   if (!J) return PIC_OK;
+  if (!j_spectral && centered) {
+    StageScope t(ctx, STAGE_OTHER, center_launches(ctx, false));
+    const float* cJ[3] = {Jnp[0], Jnp[1], Jnp[2]};
+    return center_to_yee_t<float>(ctx, cJ, J);
+  }
+  if (!j_spectral) {
+    for (int c = 0; c < 3; ++c)
+      PIC_CUDA_TRY(ctx, cudaMemcpyAsync(J[c], Jnp[c], nc * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
+    return PIC_OK;
+  }
   float* jouts[3] = {J[0], J[1], J[2]};
   return store_yee32(ctx, Jh(ctx), kKindJ, 3, jouts);
 }

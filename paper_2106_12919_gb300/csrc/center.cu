@@ -1,7 +1,8 @@
 // Finite-order centering between the nodal and Yee grids as real-space stencils
-// (Sec. 3, Eq. staggered_finite_sum, periodic).  pic_step applies the same
-// operators as their Fourier symbol inside the k-space update; these kernels
-// are the stand-alone form of the two centering rows of the step, and the
+// (Sec. 3, Eq. staggered_finite_sum, periodic).  Between its steps pic_step applies
+// the same operators as their Fourier symbol inside the k-space update; these
+// kernels are the stand-alone form of the two centering rows of the step, the
+// centering of the fields a call starts from and of the J it returns, and the
 // centering of the FDTD cycle (FP64 and FP32), which also filters its J here.
 //
 // staggered -> nodal along axis a: f_j = sum_n w_n (s[j+n-1] + s[j-n]),
@@ -125,9 +126,10 @@ void launch_window(const StencilArgs<T>& s, int axis, cudaStream_t st) {
 
 // true when a window kernel ran: below 2^20 cells their fewer threads leave SMs idle, and unaligned
 // arrays cannot take the 16-byte loads
+constexpr int64_t kWindowCells = int64_t(1) << 20;
 template <class T>
 bool launch_window_m(const StencilArgs<T>& s, int axis, cudaStream_t st) {
-  if (s.mode == 2 || s.ncell < (1 << 20)) return false;
+  if (s.mode == 2 || s.ncell < kWindowCells) return false;
   if (axis == 2 && (reinterpret_cast<uintptr_t>(s.in) | reinterpret_cast<uintptr_t>(s.out)) % 16 != 0) return false;
   switch (s.m) {
     case 1: launch_window<T, 1>(s, axis, st); return true;
@@ -189,17 +191,84 @@ pic_status apply(pic_ctx* ctx, const T* in, T* out, int mask, int mode, T* w0, T
   return PIC_OK;
 }
 
-}  // namespace
+// Small grids: one pass along its own axis for each of up to six components in one launch (launches
+// are most of their time).
+template <class T>
+struct BatchArgs {
+  const T* in[6];
+  T* out[6];
+  int axis[6];
+  int shift[3], mask[3], m[3];
+  T w[3][PIC_MAX_CENTER_M];
+  int ncell, mode;
+};
 
 template <class T>
-pic_status center_to_nodal_t(pic_ctx* ctx, const T* const F[6], T* const out[6], T* w0, T* w1) {
-  for (int c = 0; c < 6; ++c) PIC_TRY(apply<T>(ctx, F[c], out[c], kStag[c], 1, w0, w1));
+__global__ void __launch_bounds__(256) stencil_batch_kernel(BatchArgs<T> a) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= a.ncell) return;
+  const int c = blockIdx.y, x = a.axis[c];
+  const int shift = a.shift[x], mask = a.mask[x], j = (e >> shift) & mask;
+  const T* in = a.in[c] + (e - (j << shift));
+  const int d = a.mode == 1 ? -1 : 0;
+  T acc = T(0);
+#pragma unroll 4
+  for (int n = 1; n <= a.m[x]; ++n)
+    acc += a.w[x][n - 1] * (in[((j + n + d) & mask) << shift] + in[((j - n + 1 + d) & mask) << shift]);
+  a.out[c][e] = acc;
+}
+
+template <class T>
+pic_status run_batch(pic_ctx* ctx, const T* const* in, T* const* out, const int* axis, int n, int mode) {
+  BatchArgs<T> b;
+  memset(&b, 0, sizeof(b));
+  for (int c = 0; c < n; ++c) {
+    b.in[c] = in[c];
+    b.out[c] = out[c];
+    b.axis[c] = axis[c];
+  }
+  b.shift[1] = lg2i(ctx->N[2]);
+  b.shift[0] = b.shift[1] + lg2i(ctx->N[1]);
+  for (int x = 0; x < 3; ++x) {
+    b.mask[x] = (int)ctx->N[x] - 1;
+    b.m[x] = ctx->cw[x].m;
+    for (int k = 0; k < b.m[x]; ++k) b.w[x][k] = (T)ctx->cw[x].w[k];
+  }
+  b.ncell = (int)ctx->ncell;
+  b.mode = mode;
+  stencil_batch_kernel<T><<<dim3((unsigned)((ctx->ncell + 255) / 256), n), 256, 0, ctx->stream>>>(b);
+  PIC_LAUNCH_CHECK(ctx);
+  return PIC_OK;
+}
+
+}  // namespace
+
+int center_launches(const pic_ctx* ctx, bool to_nodal) {
+  return ctx->ncell < kWindowCells ? (to_nodal ? 2 : 1) : (to_nodal ? 9 : 3);
+}
+
+template <class T>
+pic_status center_to_nodal_t(pic_ctx* ctx, const T* const F[6], T* const out[6], T* w) {
+  const int64_t nc = ctx->ncell;
+  if (nc < kWindowCells) {
+    // E^x, E^y, E^z along their axis; B^x along y, B^y and B^z along x into w, then along z, z, y
+    T* const first[6] = {out[0], out[1], out[2], w, w + nc, w + 2 * nc};
+    const T* const second[3] = {w, w + nc, w + 2 * nc};
+    const int ax1[6] = {0, 1, 2, 1, 0, 0}, ax2[3] = {2, 2, 1};
+    PIC_TRY(run_batch<T>(ctx, F, first, ax1, 6, 1));
+    return run_batch<T>(ctx, second, out + 3, ax2, 3, 1);
+  }
+  for (int c = 0; c < 6; ++c) PIC_TRY(apply<T>(ctx, F[c], out[c], kStag[c], 1, w, w + nc));
   return PIC_OK;
 }
 
 template <class T>
-pic_status center_to_yee_t(pic_ctx* ctx, const T* const Jn[3], T* const out[3], T* w0, T* w1) {
-  for (int c = 0; c < 3; ++c) PIC_TRY(apply<T>(ctx, Jn[c], out[c], kStag[c], 0, w0, w1));
+pic_status center_to_yee_t(pic_ctx* ctx, const T* const Jn[3], T* const out[3]) {
+  if (ctx->ncell < kWindowCells) {
+    const int ax[3] = {0, 1, 2};
+    return run_batch<T>(ctx, Jn, out, ax, 3, 0);
+  }
+  for (int c = 0; c < 3; ++c) PIC_TRY(apply<T>(ctx, Jn[c], out[c], kStag[c], 0, (T*)nullptr, (T*)nullptr));
   return PIC_OK;
 }
 
@@ -213,17 +282,17 @@ pic_status bilinear_filter_t(pic_ctx* ctx, T* f, int passes, T* w0, T* w1) {
   return PIC_OK;
 }
 
-template pic_status center_to_nodal_t<double>(pic_ctx*, const double* const[6], double* const[6], double*, double*);
-template pic_status center_to_nodal_t<float>(pic_ctx*, const float* const[6], float* const[6], float*, float*);
-template pic_status center_to_yee_t<double>(pic_ctx*, const double* const[3], double* const[3], double*, double*);
-template pic_status center_to_yee_t<float>(pic_ctx*, const float* const[3], float* const[3], float*, float*);
+template pic_status center_to_nodal_t<double>(pic_ctx*, const double* const[6], double* const[6], double*);
+template pic_status center_to_nodal_t<float>(pic_ctx*, const float* const[6], float* const[6], float*);
+template pic_status center_to_yee_t<double>(pic_ctx*, const double* const[3], double* const[3]);
+template pic_status center_to_yee_t<float>(pic_ctx*, const float* const[3], float* const[3]);
 template pic_status bilinear_filter_t<double>(pic_ctx*, double*, int, double*, double*);
 template pic_status bilinear_filter_t<float>(pic_ctx*, float*, int, float*, float*);
 
 pic_status center_to_nodal(pic_ctx* ctx, const double* const F[6], double* const out[6]) {
-  return center_to_nodal_t<double>(ctx, F, out, ctx->Jn, ctx->Jn + ctx->ncell);
+  return center_to_nodal_t<double>(ctx, F, out, ctx->Jn);
 }
 
 pic_status center_to_yee(pic_ctx* ctx, const double* const Jn[3], double* const out[3]) {
-  return center_to_yee_t<double>(ctx, Jn, out, ctx->nodal, ctx->nodal + ctx->ncell);
+  return center_to_yee_t<double>(ctx, Jn, out);
 }

@@ -303,7 +303,7 @@ pic_status fdtd_step(pic_ctx* ctx, double* const E[3], double* const B[3], doubl
   for (int s = 0; s < nsteps; ++s) {
     {
       // E^n, B^n -> nodes (scratch: ctx->Jn, free until the deposit)
-      StageScope t(ctx, STAGE_OTHER, 9);
+      StageScope t(ctx, STAGE_OTHER, center_launches(ctx, true));
       PIC_TRY(center_to_nodal(ctx, yee, nodal));
     }
     if (ctx->sort_interval > 0 && ctx->steps_done % ctx->sort_interval == 0)
@@ -320,7 +320,7 @@ pic_status fdtd_step(pic_ctx* ctx, double* const E[3], double* const B[3], doubl
     {
       // J^{n+1/2}: optional smoothing (Sec. 2), nodes -> Yee (work arrays: ctx->nodal, free after
       // the push)
-      StageScope t(ctx, STAGE_OTHER, 3 + 9 * ctx->filter_passes);
+      StageScope t(ctx, STAGE_OTHER, center_launches(ctx, false) + 9 * ctx->filter_passes);
       for (int c = 0; c < 3 && ctx->filter_passes > 0; ++c)
         PIC_TRY(bilinear_filter_t<double>(ctx, Jn[c], ctx->filter_passes, ctx->nodal, ctx->nodal + nc));
       PIC_TRY(center_to_yee(ctx, cJn, J));

@@ -985,7 +985,12 @@ size_t tile_layout(const pic_ctx* ctx, TileArgs& t, int wx_after, bool linear) {
 
 // the layout of the context's tiles with the most CTAs per SM: the window one node shorter along x when
 // that lets more of them share one (e.g. 8 x 16 x 8 tiles: 3 -> 4 CTAs, the register limit)
+// (asked of the runtime once per context: the queries cost several microseconds each)
 pic_status choose_layout(pic_ctx* ctx, bool linear, TileArgs& t, size_t& smem, int* ctas = nullptr) {
+  if (ctx->tile_wx[linear] && !ctas) {
+    smem = tile_layout(ctx, t, ctx->tile_wx[linear], linear);
+    return PIC_OK;
+  }
   smem = tile_layout(ctx, t, 3, linear);
   TileArgs t2 = t;
   const size_t smem2 = tile_layout(ctx, t2, 2, linear);
@@ -1000,6 +1005,7 @@ pic_status choose_layout(pic_ctx* ctx, bool linear, TileArgs& t, size_t& smem, i
   int n3 = 0, n2 = 0;
   PIC_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n3, fn, kTileThreads, smem));
   PIC_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n2, fn, kTileThreads, smem2));
+  ctx->tile_wx[linear] = n2 > n3 ? 2 : 3;
   if (n2 > n3) {
     t = t2;
     smem = smem2;
@@ -1871,11 +1877,14 @@ static pic_status bin32_scratch(pic_ctx* ctx, int nsp) {
 }
 
 bool bin32_linear(pic_ctx* ctx) {
+  if (ctx->tile_linear) return ctx->tile_linear == 2;
   TileArgs t;
   size_t smem;
   int n0 = 0, n1 = 0;
-  return bin32_two_level(ctx) && choose_layout(ctx, false, t, smem, &n0) == PIC_OK && tile_layout(ctx, t, 2, true) <= (size_t)kMaxTileSmem &&
+  const bool ok = bin32_two_level(ctx) && choose_layout(ctx, false, t, smem, &n0) == PIC_OK && tile_layout(ctx, t, 2, true) <= (size_t)kMaxTileSmem &&
          tile_layout(ctx, t, 3, true) <= (size_t)kMaxTileSmem && choose_layout(ctx, true, t, smem, &n1) == PIC_OK && n1 >= n0;
+  ctx->tile_linear = ok ? 2 : 1;
+  return ok;
 }
 
 pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_species, int64_t* const* offsets,

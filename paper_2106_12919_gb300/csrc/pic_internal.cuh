@@ -158,6 +158,10 @@ struct pic_ctx {
   int bin2_species;
   uint32_t* bin2_old[PIC_MAX_BINNED_SPECIES];
   int bin2_nold;
+  // tiled FP32 push: nodes its window keeps after the tile along x for the order by cell and the class
+  // order, and whether the step uses the class order (1: no, 2: yes); 0: not chosen yet
+  int tile_wx[2];
+  int tile_linear;
   int* bin_gate;                    // FP32 form: device flag "re-bin before the next push"
   int* bin_flags;                   // FP32 binning: [0] keys out of order, [1] scatter gate (see below)
   unsigned long long* bin_outside;  // FP32 form: particles whose new cell left their tile in the last push
@@ -275,10 +279,10 @@ pic_status psatd_update_ex(pic_ctx* ctx, const double2* rn, const double2* rp, i
 // comp_kind[c]: 0..5 = Ex..Bz, 6..8 = Jx..Jz, 9 = rho.
 pic_status psatd_phase(pic_ctx* ctx, CPtr6 in, CPtr6 out, const int* comp_kind, int ncomp, int sign,
                        double scale);
-// Six field spectra, [6][nmode] each.  load: G holds the DFT of the Yee fields; EB = its paper convention,
-// and with nodal G = the DFT of the nodal fields / Ncell.  store: G = the DFT of the Yee fields of EB / Ncell.
+// Six field spectra, [6][nmode] each.  load: EB = the paper convention of G, the DFT of the Yee fields;
+// store: G = the DFT of the Yee fields of EB / Ncell.
 template <class C>
-pic_status psatd_load(pic_ctx* ctx, C* G, C* EB, bool nodal);
+pic_status psatd_load(pic_ctx* ctx, const C* G, C* EB);
 template <class C>
 pic_status psatd_store(pic_ctx* ctx, const C* EB, C* G);
 // FP32-form counterparts (FP32 spectra, FP64 tables rounded at use).
@@ -424,11 +428,12 @@ int bin32_launches(const pic_ctx* ctx, const pic_species32* sp, int n_species);
 // center.cu -------------------------------------------------------------------
 pic_status center_to_nodal(pic_ctx* ctx, const double* const F[6], double* const out[6]);
 pic_status center_to_yee(pic_ctx* ctx, const double* const Jn[3], double* const out[3]);
-// Either precision, with explicit work arrays w0, w1 (ncell elements each).
+// Either precision; w: a work array of 3 ncell elements.
 template <class T>
-pic_status center_to_nodal_t(pic_ctx* ctx, const T* const F[6], T* const out[6], T* w0, T* w1);
+pic_status center_to_nodal_t(pic_ctx* ctx, const T* const F[6], T* const out[6], T* w);
 template <class T>
-pic_status center_to_yee_t(pic_ctx* ctx, const T* const Jn[3], T* const out[3], T* w0, T* w1);
+pic_status center_to_yee_t(pic_ctx* ctx, const T* const Jn[3], T* const out[3]);
+int center_launches(const pic_ctx* ctx, bool to_nodal);  // their kernel launches
 // `passes` passes of the bilinear (1/4, 1/2, 1/4) filter along x, y, z of f in place (Sec. 2).
 template <class T>
 pic_status bilinear_filter_t(pic_ctx* ctx, T* f, int passes, T* w0, T* w1);

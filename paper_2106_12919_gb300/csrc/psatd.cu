@@ -609,19 +609,14 @@ __global__ void phase_kernel(PhaseArgs<C> p) {
 // The six field spectra between the plain DFT and the paper's convention (times the half-cell shifts h of
 // each component's staggered axes), one thread per mode for all six: the shifts and their products are
 // formed once (with one thread per component the FP64 form took 0.40 ms for 2.1 million modes, bound by
-// its FP64 operations).
-// STORE = false: eb = h in (in: the DFT of the Yee fields), and with nodal g = zeta eb nscale, the DFT of
-// the nodal gather fields (g may be in).  STORE = true: g = conj(h) eb nscale.
+// its FP64 operations).  STORE = false: out = h in; true: out = conj(h) in scale.
 template <class C>
 struct EbArgs {
   const C* in;
-  C* eb;
-  C* g;
-  const C* hs[3];                // half-cell shifts in the data precision
-  const decltype(C().x)* zt[3];  // centering symbols in the data precision
+  C* out;
+  const C* hs[3];  // half-cell shifts in the data precision
   int64_t Ny, nzh, nmode;
-  double nscale;
-  int nodal;
+  double scale;
 };
 
 template <class C, bool STORE>
@@ -631,7 +626,6 @@ __global__ void __launch_bounds__(256) eb_kernel(EbArgs<C> a) {
   if (m >= a.nmode) return;
   uint32_t ix, iy, iz;
   mode_xyz(m, (uint32_t)a.nzh, __ffsll(a.Ny) - 1, ix, iy, iz);
-  const T s = (T)a.nscale;
   C h[6];
   h[0] = a.hs[0][ix];
   h[1] = a.hs[1][iy];
@@ -643,19 +637,9 @@ __global__ void __launch_bounds__(256) eb_kernel(EbArgs<C> a) {
   h[3] = cmul(h[1], h[2]);
   h[4] = cmul(h[0], h[2]);
   h[5] = cmul(h[0], h[1]);
-  if (STORE) {
 #pragma unroll
-    for (int c = 0; c < 6; ++c) a.g[c * a.nmode + m] = cmul(a.eb[c * a.nmode + m], cscale(h[c], s));
-    return;
-  }
-  const T zx = (T)a.zt[0][ix], zy = (T)a.zt[1][iy], zz = (T)a.zt[2][iz];
-  const T z[6] = {zx * s, zy * s, zz * s, zy * zz * s, zx * zz * s, zx * zy * s};
-#pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    const C v = cmul(a.in[c * a.nmode + m], h[c]);
-    a.eb[c * a.nmode + m] = v;
-    if (a.nodal) a.g[c * a.nmode + m] = cscale(v, z[c]);
-  }
+  for (int c = 0; c < 6; ++c)
+    a.out[c * a.nmode + m] = cmul(a.in[c * a.nmode + m], STORE ? cscale(h[c], (T)a.scale) : h[c]);
 }
 
 // ---------------------------------------------------------------------------
@@ -978,43 +962,30 @@ pic_status psatd_phase32(pic_ctx* ctx, CP6<float2> in, CP6<float2> out, const in
   return psatd_phase_t<float2>(ctx, in, out, comp_kind, ncomp, sign, scale);
 }
 
-template <class C>
-static EbArgs<C> eb_args(const pic_ctx* ctx) {
+template <bool STORE, class C>
+static pic_status eb_convert(pic_ctx* ctx, const C* in, C* out) {
   EbArgs<C> a;
-  memset(&a, 0, sizeof(a));
+  a.in = in;
+  a.out = out;
   for (int k = 0; k < 3; ++k) {
-    const decltype(C().x)* unused[2];
-    tab1d(ctx, k, &unused[0], &a.zt[k], &unused[1], &a.hs[k]);
+    const decltype(C().x)* unused[3];
+    tab1d(ctx, k, &unused[0], &unused[1], &unused[2], &a.hs[k]);
   }
   a.Ny = ctx->N[1];
   a.nzh = ctx->nzh;
   a.nmode = ctx->nmode;
-  return a;
+  a.scale = 1.0 / (double)ctx->ncell;
+  eb_kernel<C, STORE><<<(unsigned)((ctx->nmode + 255) / 256), 256, 0, ctx->stream>>>(a);
+  PIC_LAUNCH_CHECK(ctx);
+  return PIC_OK;
 }
 
 template <class C>
-pic_status psatd_load(pic_ctx* ctx, C* G, C* EB, bool nodal) {
-  EbArgs<C> a = eb_args<C>(ctx);
-  a.in = a.g = G;
-  a.eb = EB;
-  a.nodal = nodal ? 1 : 0;
-  a.nscale = 1.0 / (double)ctx->ncell;
-  eb_kernel<C, false><<<(unsigned)((ctx->nmode + 255) / 256), 256, 0, ctx->stream>>>(a);
-  PIC_LAUNCH_CHECK(ctx);
-  return PIC_OK;
-}
+pic_status psatd_load(pic_ctx* ctx, const C* G, C* EB) { return eb_convert<false>(ctx, G, EB); }
 template <class C>
-pic_status psatd_store(pic_ctx* ctx, const C* EB, C* G) {
-  EbArgs<C> a = eb_args<C>(ctx);
-  a.eb = const_cast<C*>(EB);
-  a.g = G;
-  a.nscale = 1.0 / (double)ctx->ncell;
-  eb_kernel<C, true><<<(unsigned)((ctx->nmode + 255) / 256), 256, 0, ctx->stream>>>(a);
-  PIC_LAUNCH_CHECK(ctx);
-  return PIC_OK;
-}
-template pic_status psatd_load<double2>(pic_ctx*, double2*, double2*, bool);
-template pic_status psatd_load<float2>(pic_ctx*, float2*, float2*, bool);
+pic_status psatd_store(pic_ctx* ctx, const C* EB, C* G) { return eb_convert<true>(ctx, EB, G); }
+template pic_status psatd_load<double2>(pic_ctx*, const double2*, double2*);
+template pic_status psatd_load<float2>(pic_ctx*, const float2*, float2*);
 template pic_status psatd_store<double2>(pic_ctx*, const double2*, double2*);
 template pic_status psatd_store<float2>(pic_ctx*, const float2*, float2*);
 
