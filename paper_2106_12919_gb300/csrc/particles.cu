@@ -366,7 +366,8 @@ constexpr int kG64 = kT64 + 3;             // staged nodes [T0 - 1, T0 + 10)
 constexpr int kW64 = kT64 + 5;             // deposit window nodes [T0 - 2, T0 + 11)
 constexpr int kG64n = kG64 * kG64 * kG64;
 constexpr int kW64n = kW64 * kW64 * kW64;
-constexpr int kChunk64 = 2048;             // particles per CTA at most
+// particles per CTA: at most kChunk64, fewer where that leaves SMs without a chunk (chunk64)
+constexpr int kChunk64 = 2048, kChunk64Min = 256;
 // 2 CTAs of 512 threads per SM, at 64 registers with ~0.9 KB of spills per thread: measured on 4 steps of
 // 2.1 million cubic particles, push 5.47 ms; 3 CTAs of 256 at 80 registers 5.62, of 192 at 96 6.6, of 128
 // at 168 (no spills) 6.7, 2 of 256 at 128 6.1: no pipe is busy over half of the time, so warps count most
@@ -838,6 +839,7 @@ struct Tile64List {
   PushArgs a;
   int nt[3];
   int n_tiles;
+  int chunk;        // particles per chunk at most
   int32_t* tid;
   int32_t* count;   // [n_tiles], cleared
   int32_t* off;     // [n_tiles + 1]
@@ -874,7 +876,7 @@ __global__ void __launch_bounds__(1024) tile64_scan_kernel(Tile64List l) {
   for (int i = b; i < e; ++i) {
     const int n = l.count[i];
     s.x += n;
-    s.y += (n + kChunk64 - 1) / kChunk64;
+    s.y += (n + l.chunk - 1) / l.chunk;
   }
   part[threadIdx.x] = s;
   __syncthreads();
@@ -891,7 +893,7 @@ __global__ void __launch_bounds__(1024) tile64_scan_kernel(Tile64List l) {
     l.off[i] = run.x;
     l.cstart[i] = run.y;
     l.cursor[i] = run.x;
-    const int nch = (n + kChunk64 - 1) / kChunk64;
+    const int nch = (n + l.chunk - 1) / l.chunk;
     for (int k = 0; k < nch; ++k) l.ctile[run.y + k] = i;
     run.x += n;
     run.y += nch;
@@ -960,7 +962,7 @@ bool tiled64_scratch(pic_ctx* ctx, int64_t n) {
   // captured graph of an earlier call may still use them.
   if (ctx->t64_nold + 2 > kT64Old) return false;
   n = std::max(n, 2 * ctx->t64_cap);
-  const size_t nt = (size_t)tiles64(ctx), words = 2 * (size_t)n + 5 * nt + 2 + (size_t)n / kChunk64 + 1;
+  const size_t nt = (size_t)tiles64(ctx), words = 2 * (size_t)n + 5 * nt + 2 + (size_t)n / kChunk64Min + 1;
   int32_t* w = nullptr;
   int64_t* st = nullptr;
   if (cudaMalloc(&w, words * sizeof(int32_t)) != cudaSuccess ||
@@ -995,7 +997,10 @@ pic_status launch_push64_tiled(pic_ctx* ctx, const PushArgs& a) {
   l.cstart = l.off + nt + 1;
   l.tid = l.cstart + nt + 1;
   l.idx = l.tid + cap;
-  l.ctile = l.idx + cap;  // [nt + cap / kChunk64 + 1]
+  l.ctile = l.idx + cap;  // [nt + cap / kChunk64Min + 1]
+  // about two chunks per resident CTA (two per SM) of a small species; 131072 cubic particles on 32^3, in 64
+  // tiles: 64 chunks of 2048 kept 64 of 304 CTAs busy (the gradient over 20 steps there 15.16 -> 13.62 ms)
+  l.chunk = (int)std::min<int64_t>(kChunk64, std::max<int64_t>(kChunk64Min, a.n / (4 * std::max(1, ctx->nsm))));
   t.idx = l.idx;
   t.off = l.off;
   t.cstart = l.cstart;
@@ -1011,8 +1016,8 @@ pic_status launch_push64_tiled(pic_ctx* ctx, const PushArgs& a) {
   tile64_list_kernel<<<nb, 256, 0, ctx->stream>>>(l);
   PIC_LAUNCH_CHECK(ctx);
   PIC_CUDA_TRY(ctx, cudaFuncSetAttribute(push64_tile_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem64));
-  // sum over tiles of ceil(count / kChunk64) <= n_tiles + n / kChunk64: surplus CTAs return at once
-  push64_tile_kernel<P><<<(unsigned)(nt + a.n / kChunk64 + 1), kThreads64, kSmem64, ctx->stream>>>(a, t);
+  // sum over tiles of ceil(count / chunk) <= n_tiles + n / chunk: surplus CTAs return at once
+  push64_tile_kernel<P><<<(unsigned)(nt + a.n / l.chunk + 1), kThreads64, kSmem64, ctx->stream>>>(a, t);
   PIC_LAUNCH_CHECK(ctx);
   return PIC_OK;
 }
