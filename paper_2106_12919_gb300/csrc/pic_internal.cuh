@@ -38,6 +38,19 @@ __host__ __device__ __forceinline__ float2 cscale(float2 a, float s) { return ma
 __host__ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __host__ __device__ __forceinline__ float2 cmuli(float2 a) { return make_float2(-a.y, a.x); }
 
+// c + a b and c + i a b, one multiply-add per product; -a
+__device__ __forceinline__ double2 cfma(double2 c, double2 a, double2 b) {
+  c.x = fma(a.x, b.x, fma(-a.y, b.y, c.x));
+  c.y = fma(a.x, b.y, fma(a.y, b.x, c.y));
+  return c;
+}
+__device__ __forceinline__ double2 cfmai(double2 c, double2 a, double2 b) {
+  c.x = fma(-a.x, b.y, fma(-a.y, b.x, c.x));
+  c.y = fma(a.x, b.x, fma(-a.y, b.y, c.y));
+  return c;
+}
+__device__ __forceinline__ double2 cneg(double2 a) { return make_double2(-a.x, -a.y); }
+
 // Scalar / complex type pair of a precision: Real<double>::C = double2, Real<float>::C = float2.
 template <class T> struct Cplx;
 template <> struct Cplx<double> { using type = double2; };

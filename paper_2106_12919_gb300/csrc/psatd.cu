@@ -298,6 +298,62 @@ struct UpdArgs {
   int write_j;  // write the Yee-centered J back
 };
 
+// The sums of mode_update in FP64
+template <int VAR>
+__device__ __forceinline__ void fp64_update(const double* k, double c2, const double2 (&cf)[COEF_COUNT], const double2* E,
+                                            const double2* B, const double2* J, double2 rn, double2 rp, double2* En,
+                                            double2* Bn, double2* Ga, double2* Gb) {
+  using C = double2;
+  // [k] x F
+  const auto cross = [&](const C* F, C* o) {
+    constexpr int i1[3] = {1, 2, 0}, i2[3] = {2, 0, 1};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      o[a].x = fma(k[i1[a]], F[i2[a]].x, -(k[i2[a]] * F[i1[a]].x));
+      o[a].y = fma(k[i1[a]], F[i2[a]].y, -(k[i2[a]] * F[i1[a]].y));
+    }
+  };
+  C kE[3], kB[3], kJ[3];
+  cross(E, kE);
+  cross(B, kB);
+  cross(J, kJ);
+  const C TC = cf[COEF_TC], TS = cf[COEF_TS], X1 = cf[COEF_X1], X2 = cf[COEF_X2], TX3 = cf[COEF_TX3],
+          X4 = cf[COEF_X4];
+  // rho term: i (theta^2 X3 rho^n - X2 rho^{n+1})
+  const C rterm = cmuli(cfma(cmul(TX3, rn), cneg(X2), rp));
+  const C c2TS = cscale(TS, c2);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    // B^{n+1} = TC B - i TS [k]xE + i X1 [k]xJ
+    Bn[a] = cfmai(cfmai(cmul(TC, B[a]), cneg(TS), kE[a]), X1, kJ[a]);
+    // E^{n+1} = TC E + i c^2 TS [k]xB + X4 J + rterm [k]
+    En[a] = cfma(cfmai(cmul(TC, E[a]), c2TS, kB[a]), X4, J[a]);
+    En[a].x = fma(rterm.x, k[a], En[a].x);
+    En[a].y = fma(rterm.y, k[a], En[a].y);
+  }
+  if (VAR == 2) {
+    const C P1 = cf[COEF_PSI1], P2 = cf[COEF_PSI2], Y1 = cf[COEF_Y1], Y2 = cf[COEF_Y2], Y3 = cf[COEF_Y3],
+            Y4 = cf[COEF_Y4];
+    const C yr = cfma(cmul(Y3, rn), Y2, rp);
+    const C c2P2 = cscale(P2, -c2);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      // <B> = Psi1 B + i Psi2 [k]xE + i Y1 [k]xJ
+      Gb[a] = cfmai(cfmai(cmul(P1, B[a]), P2, kE[a]), Y1, kJ[a]);
+      // <E> = Psi1 E - i c^2 Psi2 [k]xB + Y4 J + (Y3 rho^n + Y2 rho^{n+1}) [k]
+      Ga[a] = cfma(cfmai(cmul(P1, E[a]), c2P2, kB[a]), Y4, J[a]);
+      Ga[a].x = fma(yr.x, k[a], Ga[a].x);
+      Ga[a].y = fma(yr.y, k[a], Ga[a].y);
+    }
+  } else {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      Ga[a] = En[a];
+      Gb[a] = Bn[a];
+    }
+  }
+}
+
 // The k-space update of one mode (Secs. 4.2-4.4): E, B in and out (paper-convention spectra),
 // J in (the DFT of the nodal deposit, or with j_yee the Yee-centered spectrum) and out (Yee-centered,
 // after the optional filter), rho^n, rho^{n+1}; G[6] out = the fields the next gather reads (E, B or
@@ -324,48 +380,54 @@ __device__ __forceinline__ void mode_update(const UpdArgs<C>& u, uint32_t ix, ui
     rn = cscale(rn, f);
     rp = cscale(rp, f);
   }
-  // [k] x F
-  auto cross = [&](const C* F, C* o) {
-    o[0] = csub(cscale(F[2], k[1]), cscale(F[1], k[2]));
-    o[1] = csub(cscale(F[0], k[2]), cscale(F[2], k[0]));
-    o[2] = csub(cscale(F[1], k[0]), cscale(F[0], k[1]));
-  };
-  C kE[3], kB[3], kJ[3];
-  cross(E, kE);
-  cross(B, kB);
-  cross(J, kJ);
-  const C TC = cf[COEF_TC], TS = cf[COEF_TS], X1 = cf[COEF_X1], X2 = cf[COEF_X2], TX3 = cf[COEF_TX3],
-          X4 = cf[COEF_X4];
-  const T c2 = (T)u.c2;
-  // rho term: i (theta^2 X3 rho^n - X2 rho^{n+1})
-  const C rterm = cmuli(csub(cmul(TX3, rn), cmul(X2, rp)));
-  C En[3], Bn[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    // B^{n+1} = TC B - i TS [k]xE + i X1 [k]xJ
-    Bn[a] = cadd(cmul(TC, B[a]), cmuli(csub(cmul(X1, kJ[a]), cmul(TS, kE[a]))));
-    // E^{n+1} = TC E + i c^2 TS [k]xB + X4 J + rterm [k]
-    En[a] = cadd(cadd(cmul(TC, E[a]), cmuli(cscale(cmul(TS, kB[a]), c2))),
-                 cadd(cmul(X4, J[a]), cscale(rterm, k[a])));
-  }
-  C Ga[3], Gb[3];
-  if (VAR == 2) {
-    const C P1 = cf[COEF_PSI1], P2 = cf[COEF_PSI2], Y1 = cf[COEF_Y1], Y2 = cf[COEF_Y2], Y3 = cf[COEF_Y3],
-            Y4 = cf[COEF_Y4];
-    const C yr = cadd(cmul(Y3, rn), cmul(Y2, rp));
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      // <B> = Psi1 B + i Psi2 [k]xE + i Y1 [k]xJ
-      Gb[a] = cadd(cmul(P1, B[a]), cmuli(cadd(cmul(P2, kE[a]), cmul(Y1, kJ[a]))));
-      // <E> = Psi1 E - i c^2 Psi2 [k]xB + Y4 J + (Y3 rho^n + Y2 rho^{n+1}) [k]
-      Ga[a] = cadd(csub(cmul(P1, E[a]), cmuli(cscale(cmul(P2, kB[a]), c2))),
-                   cadd(cmul(Y4, J[a]), cscale(yr, k[a])));
-    }
+  C En[3], Bn[3], Ga[3], Gb[3];
+  if constexpr (sizeof(T) == 8) {
+    // FP64: bound by the FP64 pipe, so every sum is one chain of multiply-adds per real component
+    // (about 290 -> 225 operations per mode of the averaged variant, whose run of 8 steps on 64x64x256
+    // went from 9.36 to 8.87 ms with it)
+    fp64_update<VAR>(k, (T)u.c2, cf, E, B, J, rn, rp, En, Bn, Ga, Gb);
   } else {
+    // [k] x F
+    auto cross = [&](const C* F, C* o) {
+      o[0] = csub(cscale(F[2], k[1]), cscale(F[1], k[2]));
+      o[1] = csub(cscale(F[0], k[2]), cscale(F[2], k[0]));
+      o[2] = csub(cscale(F[1], k[0]), cscale(F[0], k[1]));
+    };
+    C kE[3], kB[3], kJ[3];
+    cross(E, kE);
+    cross(B, kB);
+    cross(J, kJ);
+    const C TC = cf[COEF_TC], TS = cf[COEF_TS], X1 = cf[COEF_X1], X2 = cf[COEF_X2], TX3 = cf[COEF_TX3],
+            X4 = cf[COEF_X4];
+    const T c2 = (T)u.c2;
+    // rho term: i (theta^2 X3 rho^n - X2 rho^{n+1})
+    const C rterm = cmuli(csub(cmul(TX3, rn), cmul(X2, rp)));
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      Ga[a] = En[a];
-      Gb[a] = Bn[a];
+      // B^{n+1} = TC B - i TS [k]xE + i X1 [k]xJ
+      Bn[a] = cadd(cmul(TC, B[a]), cmuli(csub(cmul(X1, kJ[a]), cmul(TS, kE[a]))));
+      // E^{n+1} = TC E + i c^2 TS [k]xB + X4 J + rterm [k]
+      En[a] = cadd(cadd(cmul(TC, E[a]), cmuli(cscale(cmul(TS, kB[a]), c2))),
+                   cadd(cmul(X4, J[a]), cscale(rterm, k[a])));
+    }
+    if (VAR == 2) {
+      const C P1 = cf[COEF_PSI1], P2 = cf[COEF_PSI2], Y1 = cf[COEF_Y1], Y2 = cf[COEF_Y2], Y3 = cf[COEF_Y3],
+              Y4 = cf[COEF_Y4];
+      const C yr = cadd(cmul(Y3, rn), cmul(Y2, rp));
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        // <B> = Psi1 B + i Psi2 [k]xE + i Y1 [k]xJ
+        Gb[a] = cadd(cmul(P1, B[a]), cmuli(cadd(cmul(P2, kE[a]), cmul(Y1, kJ[a]))));
+        // <E> = Psi1 E - i c^2 Psi2 [k]xB + Y4 J + (Y3 rho^n + Y2 rho^{n+1}) [k]
+        Ga[a] = cadd(csub(cmul(P1, E[a]), cmuli(cscale(cmul(P2, kB[a]), c2))),
+                     cadd(cmul(Y4, J[a]), cscale(yr, k[a])));
+      }
+    } else {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        Ga[a] = En[a];
+        Gb[a] = Bn[a];
+      }
     }
   }
 #pragma unroll
@@ -438,7 +500,10 @@ __global__ void __launch_bounds__(256) update_kernel(UpdArgs<C> u) {
 // register caps: FP32 standard and Galilean variants 64 (4 CTAs per SM, no spills: 0.147 -> 0.128
 // ms on the laser-wakefield box), the averaged variant 128 (at 80 its larger tables spill and it
 // runs slower); FP64 128, and 255 for the averaged variant
-template <int VAR, class C, bool REAL>
+// SPLIT: one mode per thread, the mirror (blockIdx.y >> 1, blockIdx.y & 1) of its entry (a template
+// parameter: the loop bounds as run-time values cost the FP32 form spills at its register caps, 0.140
+// instead of 0.129 ms per step on 128x128x512)
+template <int VAR, class C, bool REAL, bool SPLIT>
 __global__ void __launch_bounds__(256, sizeof(C) == 8 ? (VAR == 2 ? 2 : 4) : (VAR == 2 ? 1 : 2))
     update_quad_kernel(UpdArgs<C> u) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -469,16 +534,19 @@ __global__ void __launch_bounds__(256, sizeof(C) == 8 ? (VAR == 2 ? 2 : 4) : (VA
   }
   const uint32_t Nx = (uint32_t)u.coef.nx, Ny = (uint32_t)u.coef.ny;
   const int nmx = (qx == 0 || 2 * qx == Nx) ? 1 : 2, nmy = (qy == 0 || 2 * qy == Ny) ? 1 : 2;
-  // gridDim.y == 4: this thread takes the mirror (blockIdx.y >> 1, blockIdx.y & 1) only
-  const bool split = gridDim.y == 4;
-  const int a0 = split ? blockIdx.y >> 1 : 0, a1 = split ? min(nmx, a0 + 1) : nmx;
-  const int b0 = split ? blockIdx.y & 1 : 0, b1 = split ? min(nmy, b0 + 1) : nmy;
-  for (int a = a0; a < a1; ++a) {
-    const uint32_t ix = a ? Nx - qx : qx;
-    for (int b = b0; b < b1; ++b) {
-      const uint32_t iy = b ? Ny - qy : qy;
-      const int64_t m = ((int64_t)ix * Ny + iy) * nzh + iz;
-      update_one<VAR>(u, m, ix, iy, iz, cf);
+  if constexpr (SPLIT) {
+    const int a = blockIdx.y >> 1, b = blockIdx.y & 1;
+    if (a >= nmx || b >= nmy) return;
+    const uint32_t ix = a ? Nx - qx : qx, iy = b ? Ny - qy : qy;
+    update_one<VAR>(u, ((int64_t)ix * Ny + iy) * nzh + iz, ix, iy, iz, cf);
+  } else {
+    for (int a = 0; a < nmx; ++a) {
+      const uint32_t ix = a ? Nx - qx : qx;
+      for (int b = 0; b < nmy; ++b) {
+        const uint32_t iy = b ? Ny - qy : qy;
+        const int64_t m = ((int64_t)ix * Ny + iy) * nzh + iz;
+        update_one<VAR>(u, m, ix, iy, iz, cf);
+      }
     }
   }
 }
@@ -901,9 +969,15 @@ pic_status psatd_update_t(pic_ctx* ctx, C* EB, C* J, const C* rn, const C* rp, C
     const bool split = ctx->nq < (int64_t)2 * 256 * ctx->nsm;
     if (split) bs = 64;
     const dim3 nb((unsigned)((ctx->nq + bs - 1) / bs), split ? 4 : 1);
-    if (avg) update_quad_kernel<2, C, false><<<nb, bs, 0, ctx->stream>>>(u);
-    else if (ctx->coefq_real) update_quad_kernel<0, C, true><<<nb, bs, 0, ctx->stream>>>(u);
-    else update_quad_kernel<0, C, false><<<nb, bs, 0, ctx->stream>>>(u);
+    if (split) {
+      if (avg) update_quad_kernel<2, C, false, true><<<nb, bs, 0, ctx->stream>>>(u);
+      else if (ctx->coefq_real) update_quad_kernel<0, C, true, true><<<nb, bs, 0, ctx->stream>>>(u);
+      else update_quad_kernel<0, C, false, true><<<nb, bs, 0, ctx->stream>>>(u);
+    } else {
+      if (avg) update_quad_kernel<2, C, false, false><<<nb, bs, 0, ctx->stream>>>(u);
+      else if (ctx->coefq_real) update_quad_kernel<0, C, true, false><<<nb, bs, 0, ctx->stream>>>(u);
+      else update_quad_kernel<0, C, false, false><<<nb, bs, 0, ctx->stream>>>(u);
+    }
   } else {
     const unsigned nb = (unsigned)((ctx->nmode + bs - 1) / bs);
     if (avg) update_kernel<2, C><<<nb, bs, 0, ctx->stream>>>(u);
