@@ -999,7 +999,7 @@ pic_status launch_push64_tiled(pic_ctx* ctx, const PushArgs& a) {
   l.idx = l.tid + cap;
   l.ctile = l.idx + cap;  // [nt + cap / kChunk64Min + 1]
   // about two chunks per resident CTA (two per SM) of a small species; 131072 cubic particles on 32^3, in 64
-  // tiles: 64 chunks of 2048 kept 64 of 304 CTAs busy (the gradient over 20 steps there 15.16 -> 13.62 ms)
+  // tiles: 64 chunks of 2048 kept 64 of 304 CTAs busy (the gradient over 8 steps there 15.16 -> 13.62 ms)
   l.chunk = (int)std::min<int64_t>(kChunk64, std::max<int64_t>(kChunk64Min, a.n / (4 * std::max(1, ctx->nsm))));
   t.idx = l.idx;
   t.off = l.off;

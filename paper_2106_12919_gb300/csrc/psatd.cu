@@ -383,7 +383,7 @@ __device__ __forceinline__ void mode_update(const UpdArgs<C>& u, uint32_t ix, ui
   C En[3], Bn[3], Ga[3], Gb[3];
   if constexpr (sizeof(T) == 8) {
     // FP64: bound by the FP64 pipe, so every sum is one chain of multiply-adds per real component
-    // (about 290 -> 225 operations per mode of the averaged variant, whose run of 8 steps on 64x64x256
+    // (about 290 -> 225 operations per mode of the averaged variant, whose run of 4 steps on 64x64x256
     // went from 9.36 to 8.87 ms with it)
     fp64_update<VAR>(k, (T)u.c2, cf, E, B, J, rn, rp, En, Bn, Ga, Gb);
   } else {
