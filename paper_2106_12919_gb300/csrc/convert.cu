@@ -27,27 +27,60 @@ struct SplitArgs {
   int64_t n;
 };
 
-// Both kernels move 104 bytes per particle and were bound by 64-bit integer divisions by the grid sizes
-// and, the join, by FP64-pipe conversions: 68.1 million particles 2.26 (split) and 2.45 ms (join).
+// Both kernels move 104 bytes per particle, 15.5 ps at the copy bandwidth.  They were bound by the FP64
+// pipe: floors, additions and conversions between formats, at 1.7 to 2 per clock and SM, took 34 (split) and
+// 32 ps (join, 68.1 million particles).  On the bit patterns, with one FP64 product per coordinate left,
+// 19.5 and 20.9 ps (16.8 million).
+
+// (float)v, rounded to nearest even: normal results and zeros without the FP64 pipe
+__device__ __forceinline__ float narrow(double v) {
+  const uint64_t b = (uint64_t)__double_as_longlong(v), m = b & 0x7fffffffffffffffull;
+  const uint32_t sign = (uint32_t)(b >> 63) << 31;
+  if (m == 0ull) return __uint_as_float(sign);
+  if ((uint32_t)(m >> 52) - 897u >= 253u) return __double2float_rn(v);  // (the result's exponent field: 1 .. 253)
+  const uint64_t r = m - (896ull << 52);
+  return __uint_as_float((uint32_t)((r + 0x0fffffffull + ((r >> 29) & 1ull)) >> 29) | sign);
+}
+
+// cell (not wrapped) and offset of t = x / dx: floor(t), and t - floor(t) rounded to FP32
+__device__ __forceinline__ int split_cell(double t, float& f) {
+  const uint64_t b = (uint64_t)__double_as_longlong(t);
+  const int sh = 1075 - (int)(b >> 52);                      // t = m 2^-sh
+  const uint64_t m = (b & 0xfffffffffffffull) | (1ull << 52);
+  const int i = sh > 52 ? 0 : (int)(m >> (sh & 63));
+  const uint64_t r = sh > 52 ? m : m & ((1ull << (sh & 63)) - 1ull);
+  const int lz = __clzll((long long)r), ef = 190 - lz - sh;  // the offset's exponent field
+  if (sh < 22 || ef < 1 || r == 0ull) {  // t < 0, t >= 2^31 or not finite (sh < 22, the sign being part of it); tiny or zero offsets
+    if (sh >= 22 && r == 0ull) {
+      f = 0.0f;
+      return i;
+    }
+    const double c = floor(t);
+    f = __double2float_rn(t - c);
+    return (int)(int64_t)c;
+  }
+  const uint64_t n = r << lz;
+  const uint32_t m24 = (uint32_t)(n >> 40);
+  const uint64_t rest = n << 24;
+  const uint32_t up = rest > (1ull << 63) || (rest == (1ull << 63) && (m24 & 1u)) ? 1u : 0u;
+  f = __uint_as_float(((uint32_t)ef << 23) + (m24 & 0x7fffffu) + up);
+  return i;
+}
+
 __global__ void split_kernel(SplitArgs a) {
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < a.n; p += (int64_t)gridDim.x * blockDim.x) {
     int idx[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const double t = __dmul_rn(a.x[d][p], a.inv_dx[d]);
-      const double b = floor(t);
-      float f = __double2float_rn(t - b);
-      int64_t i = (int64_t)b;
-      if (f == 1.0f) {
-        f = 0.0f;
-        i += 1;
-      }
-      idx[d] = (int)i & a.mask[d];
+      float f;
+      int i = split_cell(__dmul_rn(a.x[d][p], a.inv_dx[d]), f);
+      if (f == 1.0f) f = 0.0f, ++i;
+      idx[d] = i & a.mask[d];
       a.f[d][p] = f;
-      a.u32[d][p] = __double2float_rn(a.u[d][p]);
+      a.u32[d][p] = narrow(a.u[d][p]);
     }
     a.cell[p] = (((idx[0] << a.sy) + idx[1]) << a.sz) + idx[2];
-    a.w32[p] = __double2float_rn(a.w[p]);
+    a.w32[p] = narrow(a.w[p]);
     if (a.id_out) a.id_out[p] = a.id_in[p];
   }
 }
@@ -76,13 +109,24 @@ __device__ __forceinline__ double widen(float f) {
   return __longlong_as_double((int64_t)(m | ((uint64_t)(b >> 31) << 63)));
 }
 
+// i + f for a cell 0 <= i < 1024 and an offset f in [0, 1): exact and without the FP64 pipe from f = 2^-20
+// (the sum's lowest bit is then 53 or fewer below its highest) and for f = 0
+__device__ __forceinline__ double cell_plus(int i, float f) {
+  const uint32_t b = __float_as_uint(f), e = b >> 23;
+  if ((uint32_t)i >= 1024u || (b != 0u && e - 107u >= 20u)) return (double)i + widen(f);
+  const uint64_t s = ((uint64_t)(uint32_t)i << 52) + (b == 0u ? 0ull : (uint64_t)((b & 0x7fffffu) | 0x800000u) << (e - 98u & 63u));
+  if (s == 0ull) return 0.0;
+  const int lz = __clzll((long long)s);
+  return __longlong_as_double((int64_t)(((uint64_t)(1034 - lz) << 52) | (s << lz << 1 >> 12)));
+}
+
 __global__ void join_kernel(JoinArgs a) {
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < a.n; p += (int64_t)gridDim.x * blockDim.x) {
     const int c = a.cell[p];
     const int idx[3] = {c >> (a.sy + a.sz), (c >> a.sz) & a.mask[1], c & a.mask[2]};
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      a.x[d][p] = __dmul_rn((double)idx[d] + widen(a.f[d][p]), a.dx[d]);
+      a.x[d][p] = __dmul_rn(cell_plus(idx[d], a.f[d][p]), a.dx[d]);
       a.u[d][p] = widen(a.u32[d][p]);
     }
     a.w[p] = widen(a.w32[p]);

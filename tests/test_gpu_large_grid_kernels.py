@@ -173,6 +173,49 @@ def test_widening_of_special_values():
         np.testing.assert_array_equal(got[ok].view(np.int64), want[ok].view(np.int64))
 
 
+def test_splitting_of_special_values():
+    """FP64 -> FP32 on the bit patterns: ties, results that are subnormal, overflow or are not finite, offsets
+    down to 2^-1074, positions outside the box; and back (offsets below 2^-20 included), bit for bit."""
+    import torch
+    from paper_2106_12919_gb300 import pic
+    shape, dx = (8, 16, 1024), (1.0, 0.25, 0.04)
+    ctx = ctx32(_params(shape, dx=dx))
+    rng = np.random.default_rng(9)
+    k = np.arange(4000)
+    pos = [np.where(k % 4 == 0, (k % shape[a]) + 2.0 ** -(k % 70), np.where(
+        k % 4 == 1, np.nextafter((k % shape[a]) + 1.0, 0.0), np.where(
+            k % 4 == 2, 2.0 ** -(k * 0.27), (k % shape[a]) + (2 * (k % 512) + 1) * 2.0 ** -25))) * dx[a] for a in range(3)]
+    pos = [np.clip(v, 0.0, np.nextafter(shape[a] * dx[a], 0.0)) for a, v in enumerate(pos)]
+    u = rng.normal(size=k.size) * 10.0 ** rng.uniform(-46, 39, k.size)
+    u[:500] = (1.0 + k[:500] * 2.0 ** -24) * 2.0 ** (k[:500] % 250 - 125.0)
+    u[500:512] = [0.0, -0.0, np.inf, -np.inf, np.nan, 1e300, -1e300, 1e-300, 2.0 ** -150, 3.4028235677973366e38, 1e-45, 5e-324]
+    dev = [to_dev(v) for v in (*pos, u, -u, u[::-1], u)]
+    s = pic.Species32.from_positions(ctx, *dev, -1.0, 1.0)
+    ctx.sync()
+    ref = [particles.cell_offset_split(v, dx[a], shape[a]) for a, v in enumerate(pos)]
+    np.testing.assert_array_equal(to_host(s.cell), particles.linear_cell(ref[0][0], ref[1][0], ref[2][0], shape))
+    with np.errstate(all="ignore"):
+        want32 = [v.astype(np.float32) for v in (u, -u, u[::-1], u)]
+    for got, want in zip((s.fx, s.fy, s.fz, s.ux, s.uy, s.uz, s.w), [r[1] for r in ref] + want32):
+        got = to_host(got)
+        ok = ~np.isnan(want)
+        np.testing.assert_array_equal(np.isnan(got), ~ok)
+        np.testing.assert_array_equal(got[ok].view(np.uint32), want[ok].view(np.uint32))
+    b = ctx.species32_to_species(s)
+    ctx.sync()
+    for a, got in enumerate((b.x, b.y, b.z)):
+        np.testing.assert_array_equal(to_host(got), particles.cell_offset_join(ref[a][0], ref[a][1], dx[a]))
+    # outside the box: the cell wraps, the offset is that of the position
+    far = [np.array([-0.3, -17.6, 1e9 + 0.5, 3e12, -0.0]) * dx[a] for a in range(3)]
+    z = to_dev(np.zeros(5))
+    s = pic.Species32.from_positions(ctx, *[to_dev(v) for v in far], z, z, z, z, -1.0, 1.0)
+    ctx.sync()
+    for a, got in enumerate((s.fx, s.fy, s.fz)):
+        t = far[a] * (1.0 / dx[a])
+        f = (t - np.floor(t)).astype(np.float32)
+        np.testing.assert_array_equal(to_host(got), np.where(f == 1.0, np.float32(0.0), f))
+
+
 @pytest.mark.parametrize("order", [1, 2, 3])
 @pytest.mark.parametrize("kind", ["sorted", "random", "faces", "peak", "spread", "ramp", "inf"])
 def test_deposit_rho32_windows(order, kind):
