@@ -40,9 +40,8 @@ struct AdjArgs {
 template <int P>
 __device__ __forceinline__ void shape_d(double x, double inv, int& lo, double* S, double* D) {
   const double t = __dmul_rn(x, inv);
-  const double base = (P == 2) ? floor(__dadd_rn(t, 0.5)) : floor(t);
-  const double d = t - base;
-  const int b = (int)base;
+  int b;
+  const double d = t - floor_cell(P == 2 ? __dadd_rn(t, 0.5) : t, b);
   if (P == 1) {
     lo = b;
     S[0] = 1.0 - d;

@@ -41,11 +41,8 @@ struct PushArgs {
 template <int P>
 __device__ __forceinline__ void shape(double x, double inv, int mask, int& lo, double* S, double off = 0.0) {
   const double t = __dmul_rn(x, inv) - off;
-  double base;
-  if (P == 2) base = floor(__dadd_rn(t, 0.5));
-  else base = floor(t);
-  const double d = t - base;
-  const int b = (int)base;
+  int b;
+  const double d = t - floor_cell(P == 2 ? __dadd_rn(t, 0.5) : t, b);
   if (P == 1) {
     lo = b;
     S[0] = 1.0 - d;
@@ -58,11 +55,12 @@ __device__ __forceinline__ void shape(double x, double inv, int mask, int& lo, d
     S[2] = 0.5 * c * c;
   } else {
     lo = b - 1;
-    const double e = 1.0 - d, d2 = d * d, d3 = d2 * d;
-    S[0] = e * e * e * (1.0 / 6.0);
-    S[1] = (4.0 - 6.0 * d2 + 3.0 * d3) * (1.0 / 6.0);
-    S[2] = (1.0 + 3.0 * d + 3.0 * d2 - 3.0 * d3) * (1.0 / 6.0);
-    S[3] = d3 * (1.0 / 6.0);
+    // the inner weights as 2/3 + d^2 (d/2 - 1) and its mirror image
+    const double e = 1.0 - d, d2 = d * d, e2 = e * e;
+    S[0] = e2 * (e * (1.0 / 6.0));
+    S[1] = fma(d2, fma(0.5, d, -1.0), 2.0 / 3.0);
+    S[2] = fma(e2, fma(0.5, e, -1.0), 2.0 / 3.0);
+    S[3] = d2 * (d * (1.0 / 6.0));
   }
   (void)mask;
 }
@@ -84,12 +82,12 @@ __device__ __forceinline__ void push_u(const PushArgs& a, int64_t p, const doubl
   const double tx = k * f[3] * igm, ty = k * f[4] * igm, tz = k * f[5] * igm;
   const double s2 = 2.0 / (1.0 + tx * tx + ty * ty + tz * tz);
   const double sx = s2 * tx, sy = s2 * ty, sz = s2 * tz;
-  const double upx = umx + (umy * tz - umz * ty);
-  const double upy = umy + (umz * tx - umx * tz);
-  const double upz = umz + (umx * ty - umy * tx);
-  ux = umx + (upy * sz - upz * sy) + k * f[0];
-  uy = umy + (upz * sx - upx * sz) + k * f[1];
-  uz = umz + (upx * sy - upy * sx) + k * f[2];
+  const double upx = fma(umy, tz, fma(-umz, ty, umx));
+  const double upy = fma(umz, tx, fma(-umx, tz, umy));
+  const double upz = fma(umx, ty, fma(-umy, tx, umz));
+  ux = fma(upy, sz, fma(-upz, sy, fma(k, f[0], umx)));
+  uy = fma(upz, sx, fma(-upx, sz, fma(k, f[1], umy)));
+  uz = fma(upx, sy, fma(-upy, sx, fma(k, f[2], umz)));
 }
 
 // x in [0, L) after a move of less than a period; the comparisons are on the bit patterns (of positive

@@ -38,6 +38,26 @@ __host__ __device__ __forceinline__ float2 cscale(float2 a, float s) { return ma
 __host__ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __host__ __device__ __forceinline__ float2 cmuli(float2 a) { return make_float2(-a.y, a.x); }
 
+// floor(t), also as an integer, on the bit pattern for 0 <= t < 2^31: rounding and conversion instructions
+// take the FP64 pipe, which bounds the FP64 particle kernels (with the pushers' cross products as chains of
+// multiply-adds: 10 steps of 262107 linear particles on 32^3 2.48 -> 2.42 ms)
+__device__ __forceinline__ double floor_cell(double t, int& i) {
+  const long long b = __double_as_longlong(t);
+  const int e = (int)(b >> 52);  // sign and exponent
+  if (e < 0 || e > 1053) {       // t < 0, t >= 2^31 or not finite
+    const double f = floor(t);
+    i = (int)f;
+    return f;
+  }
+  if (e < 1023) {
+    i = 0;
+    return 0.0;
+  }
+  const int sh = 1075 - e;
+  i = (int)(((b & 0xfffffffffffffll) | (1ll << 52)) >> sh);
+  return __longlong_as_double(b >> sh << sh);
+}
+
 // c + a b and c + i a b, one multiply-add per product; -a
 __device__ __forceinline__ double2 cfma(double2 c, double2 a, double2 b) {
   c.x = fma(a.x, b.x, fma(-a.y, b.y, c.x));
