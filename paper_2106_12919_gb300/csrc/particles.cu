@@ -371,6 +371,9 @@ constexpr int kChunk64 = 2048, kChunk64Min = 256;
 // at 168 (no spills) 6.7, 2 of 256 at 128 6.1: no pipe is busy over half of the time, so warps count most
 constexpr int kThreads64 = 512;
 constexpr int kMinTiled = 16;
+// rho by itself (pic_deposit_rho) from this many particles: 131072 cubic ones take 53 us this way and 55 one
+// by one (bound by the FP64 pipe: 120 operations each), 1.06 million 189 and 294, 2.1 million 277 and 539
+constexpr int64_t kMinRho64 = 1 << 18;
 constexpr int kB64 = kW64 - 2;             // first nodes of shape blocks in the window (node_bounds)
 constexpr int kB64n = kB64 * kB64 * kB64;
 constexpr size_t kWin64 = (size_t)kW64n * 4 * 8;   // >= the staged fields, kG64n * 48
@@ -534,8 +537,8 @@ __device__ __forceinline__ void deposit56(uint32_t* win, int c0, const int64_t* 
 // quadratic one) of those of the blocks that reach it.  The bound decides the sums' unit: from the
 // chunk's total times the largest weight it is 30 times larger at 2 particles per cell, and J of random
 // momenta came out 5.4e-15 off the exact one; with this 1.8e-15, as with FP64 atomics.
-// tmp: 4 kW64 kB64 (kB64 + kW64) floats.  Called by the whole CTA.
-template <int P>
+// tmp: 4 kW64 kB64 (kB64 + kW64) floats.  Components C0 .. 3 only.  Called by the whole CTA.
+template <int P, int C0>
 __device__ __forceinline__ void node_bounds(const float* blk, float* tmp, unsigned* out) {
   // the sum over the slots s of the largest weight in slot s times v[(n - s) * stride], n - s in [0, kB64)
   const auto line = [](const float* v, int n, int stride) {
@@ -550,17 +553,17 @@ __device__ __forceinline__ void node_bounds(const float* blk, float* tmp, unsign
   constexpr int B2 = kB64 * kB64;
   float* X = tmp;                    // [4][kW64][kB64][kB64]
   float* Y = tmp + 4 * kW64 * B2;    // [4][kW64][kW64][kB64]
-  for (int e = threadIdx.x; e < 4 * kW64 * B2; e += kThreads64) {
+  for (int e = threadIdx.x + C0 * kW64 * B2; e < 4 * kW64 * B2; e += kThreads64) {
     const int yz = e % B2, n = e / B2 % kW64, c = e / B2 / kW64;
     X[e] = line(blk + c * kB64n + yz, n, B2);
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < 4 * kW64 * kW64 * kB64; e += kThreads64) {
+  for (int e = threadIdx.x + C0 * kW64 * kW64 * kB64; e < 4 * kW64 * kW64 * kB64; e += kThreads64) {
     const int z = e % kB64, n = e / kB64 % kW64, cx = e / kB64 / kW64;
     Y[e] = line(X + cx * B2 + z, n, kB64);
   }
   __syncthreads();
-  for (int c = 0; c < 4; ++c) {
+  for (int c = C0; c < 4; ++c) {
     float mx = 0.0f;
     for (int e = threadIdx.x; e < kW64n; e += kThreads64)
       mx = fmaxf(mx, line(Y + (c * kW64 * kW64 + e / kW64) * kB64, e % kW64, 1));
@@ -571,7 +574,8 @@ __device__ __forceinline__ void node_bounds(const float* blk, float* tmp, unsign
 }
 static_assert((size_t)4 * kW64 * kB64 * (kB64 + kW64) * sizeof(float) <= kWin64, "node_bounds");
 
-template <int P>
+// RHO: only rho of the particles as they are (no fields, no push, no J; see kMinRho64)
+template <int P, bool RHO>
 __global__ void __launch_bounds__(kThreads64, 2) push64_tile_kernel(const __grid_constant__ PushArgs a, Tile64Args t) {
   constexpr int NS = P + 1;
   extern __shared__ __align__(16) unsigned char smraw64[];
@@ -605,7 +609,7 @@ __global__ void __launch_bounds__(kThreads64, 2) push64_tile_kernel(const __grid
   for (int e = threadIdx.x; e < 4 * kB64n; e += kThreads64) s_blk[e] = 0.0f;  // (synchronised below)
   // [3][kG64n] pairs of components: first the doubles, then (h, l) limbs of each in their place
   int4* fld = reinterpret_cast<int4*>(smraw64);
-  if (!alone) {
+  if (!RHO && !alone) {
     unsigned mx[6] = {0u, 0u, 0u, 0u, 0u, 0u};
     for (int e = threadIdx.x; e < kG64n; e += kThreads64) {
       const int k = e % kG64, r = e / kG64, j = r % kG64, i = r / kG64;
@@ -631,7 +635,7 @@ __global__ void __launch_bounds__(kThreads64, 2) push64_tile_kernel(const __grid
     for (int j = threadIdx.x; j < cnt; j += kThreads64) push_particle_alone<P>(a, t.idx[p0 + j]);
     return;
   }
-  for (int e = threadIdx.x; e < kG64n; e += kThreads64) {
+  for (int e = threadIdx.x; !RHO && e < kG64n; e += kThreads64) {
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       const double2 v = reinterpret_cast<double2*>(fld)[q * kG64n + e];
@@ -646,7 +650,33 @@ __global__ void __launch_bounds__(kThreads64, 2) push64_tile_kernel(const __grid
   const int q = (cnt + s - 1) / s;
   // phase 1: gather, push, move; positions and amounts of the deposits go to the stash
   unsigned amax[4] = {0u, 0u, 0u, 0u};
-  for (int jj = threadIdx.x; jj < q * s; jj += kThreads64) {
+  for (int jj = threadIdx.x; RHO && jj < q * s; jj += kThreads64) {
+    const int row = jj / q, pr = (jj - row * q) * s + row;
+    if (pr >= cnt) continue;
+    const int64_t p = t.idx[p0 + pr];
+    int64_t* st = t.stash + p0 + pr;
+    const double x[3] = {a.x[p], a.y[p], a.z[p]}, qw = a.w[p] * a.qw_scale;
+    bool ok = qw == 0.0 || (exponent_of(qw) >= 200 && exponent_of(qw) < 1900);
+    int b[3];
+    int64_t d[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      ok = ok && split56<P>(x[c], a.inv_dx[c], b[c], d[c]);
+      b[c] = ok ? (b[c] - T0[c] + 1) & a.mask[c] : 0;  // first node of the block in the window
+      ok = ok && b[c] + NS <= kW64;
+    }
+    st[0] = ok ? 0 : -1;
+    if (!ok) {
+      push_particle_alone<P>(a, p);
+      continue;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) st[(3 + c) * t.cap] = ((int64_t)b[c] << 56) | d[c];
+    st[9 * t.cap] = __double_as_longlong(qw);
+    amax[3] = max(amax[3], (unsigned)exponent_of(qw));
+    atomicAdd(&s_blk[3 * kB64n + (b[0] * kB64 + b[1]) * kB64 + b[2]], fabsf((float)qw));
+  }
+  for (int jj = threadIdx.x; !RHO && jj < q * s; jj += kThreads64) {
     const int row = jj / q, pr = (jj - row * q) * s + row;
     if (pr >= cnt) continue;
     const int64_t slot = p0 + pr, p = t.idx[slot];
@@ -771,7 +801,7 @@ __global__ void __launch_bounds__(kThreads64, 2) push64_tile_kernel(const __grid
   __syncthreads();
   // the units of the four sums, 2^(ref - 1080): every node's sum < 2^63 units (the bound has 1 % to spare); where the FP32 bound is
   // out of that type's range, from the count of particles
-  node_bounds<P>(s_blk, reinterpret_cast<float*>(smraw64), s_bound);
+  node_bounds<P, RHO ? 3 : 0>(s_blk, reinterpret_cast<float*>(smraw64), s_bound);
   int ref[4];
   {
 #pragma unroll
@@ -810,10 +840,12 @@ __global__ void __launch_bounds__(kThreads64, 2) push64_tile_kernel(const __grid
     };
     pos[0] = st[0];
     if (pos[0] < 0) continue;
-    pos[1] = st[t.cap];
-    pos[2] = st[2 * t.cap];
-    amounts(0, 3);
-    deposit56<P, 3>(win, 0, pos, am, l, lz);
+    if constexpr (!RHO) {
+      pos[1] = st[t.cap];
+      pos[2] = st[2 * t.cap];
+      amounts(0, 3);
+      deposit56<P, 3>(win, 0, pos, am, l, lz);
+    }
 #pragma unroll
     for (int c = 0; c < 3; ++c) pos[c] = st[(3 + c) * t.cap];
     amounts(3, 1);
@@ -825,7 +857,7 @@ __global__ void __launch_bounds__(kThreads64, 2) push64_tile_kernel(const __grid
     const int k = e % kW64, r = e / kW64, j = r % kW64, i = r / kW64;
     const int o = (((T0[0] - 2 + i) & a.mask[0]) * Ny + ((T0[1] - 2 + j) & a.mask[1])) * Nz + ((T0[2] - 2 + k) & a.mask[2]);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = RHO ? 3 : 0; c < 4; ++c) {
       const int64_t v = (int64_t)(((uint64_t)win[(4 + c) * kW64n + e] << 32) | win[c * kW64n + e]);
       if (v != 0) atomicAdd(dst[c] + o, from_fixed(v, ref[c] - 1080));
     }
@@ -979,7 +1011,7 @@ bool tiled64_scratch(pic_ctx* ctx, int64_t n) {
   return true;
 }
 
-template <int P>
+template <int P, bool RHO>
 pic_status launch_push64_tiled(pic_ctx* ctx, const PushArgs& a) {
   const int nt = tiles64(ctx);
   const int64_t cap = ctx->t64_cap;
@@ -1013,9 +1045,9 @@ pic_status launch_push64_tiled(pic_ctx* ctx, const PushArgs& a) {
   PIC_LAUNCH_CHECK(ctx);
   tile64_list_kernel<<<nb, 256, 0, ctx->stream>>>(l);
   PIC_LAUNCH_CHECK(ctx);
-  PIC_CUDA_TRY(ctx, cudaFuncSetAttribute(push64_tile_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem64));
+  PIC_CUDA_TRY(ctx, cudaFuncSetAttribute(push64_tile_kernel<P, RHO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem64));
   // sum over tiles of ceil(count / chunk) <= n_tiles + n / chunk: surplus CTAs return at once
-  push64_tile_kernel<P><<<(unsigned)(nt + a.n / l.chunk + 1), kThreads64, kSmem64, ctx->stream>>>(a, t);
+  push64_tile_kernel<P, RHO><<<(unsigned)(nt + a.n / l.chunk + 1), kThreads64, kSmem64, ctx->stream>>>(a, t);
   PIC_LAUNCH_CHECK(ctx);
   return PIC_OK;
 }
@@ -1023,7 +1055,9 @@ pic_status launch_push64_tiled(pic_ctx* ctx, const PushArgs& a) {
 pic_status launch_push(pic_ctx* ctx, const PushArgs& a) {
   if (a.n == 0) return PIC_OK;
   if (a.gather && use_tiled64(ctx, a.n) && tiled64_scratch(ctx, a.n))
-    return ctx->shape_order == 2 ? launch_push64_tiled<2>(ctx, a) : launch_push64_tiled<3>(ctx, a);
+    return ctx->shape_order == 2 ? launch_push64_tiled<2, false>(ctx, a) : launch_push64_tiled<3, false>(ctx, a);
+  if (!a.gather && use_tiled64(ctx, a.n) && a.n >= kMinRho64 && tiled64_scratch(ctx, a.n))
+    return ctx->shape_order == 2 ? launch_push64_tiled<2, true>(ctx, a) : launch_push64_tiled<3, true>(ctx, a);
   const int bs = 256;
   const unsigned nb = (unsigned)((a.n + bs - 1) / bs);
   if (a.gather && ctx->cycle == PIC_CYCLE_STAGGERED) {

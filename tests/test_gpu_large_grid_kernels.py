@@ -289,3 +289,40 @@ def test_tiled64_chunk_sizes(n):
     order = np.argsort(to_host(d.id))
     for k in ("ux", "uy", "uz"):
         assert np.max(np.abs(to_host(getattr(d, k))[order] - ref[k])) < 1e-12 * np.max(np.abs(ref[k]))
+
+
+@pytest.mark.parametrize("order", [2, 3])
+@pytest.mark.parametrize("kind", ["below", "first", "sorted", "faces", "spread", "outside", "inf"])
+def test_deposit_rho_tiled64(order, kind):
+    """FP64 rho by itself, on both sides of the count from which it is summed per tile, against the oracle."""
+    import torch
+    shape, dx = (16, 16, 32), (0.5, 1.0, 0.25)
+    ctx = context_for(_params(shape, dx=dx, shape_order=order))
+    rng = np.random.default_rng(order)
+    n = 2 ** 18 - 1 if kind == "below" else 2 ** 18 if kind == "first" else 300007
+    s = {k: rng.uniform(0, shape[a] * dx[a], n) for a, k in enumerate("xyz")}
+    s.update({k: np.zeros(n) for k in ("ux", "uy", "uz")}, w=rng.uniform(0.5, 1.5, n), q=-1.0, m=1.0)
+    if kind == "sorted":
+        s["x"].sort()
+    elif kind == "faces":
+        for a, k in enumerate("xyz"):
+            s[k][a::3] = rng.integers(0, shape[a], s[k][a::3].size) * dx[a]
+            s[k][:50], s[k][50:100] = np.nextafter(shape[a] * dx[a], 0.0), 0.5 * dx[a]
+    elif kind == "spread":
+        s["w"] *= 10.0 ** rng.uniform(-8, 0, n)
+    elif kind == "outside":
+        for a, k in enumerate("xyz"):
+            s[k][:500] += shape[a] * dx[a] * rng.integers(-1, 2, 500)
+    elif kind == "inf":
+        s["w"][n // 2] = np.inf
+    (d,) = species_to_dev([s])
+    rho = torch.empty(ctx.ncell, dtype=torch.float64, device="cuda")
+    ctx.deposit_rho([d], rho)
+    ctx.sync()
+    got = to_host(rho).reshape(shape)
+    ok = np.isfinite(got)
+    assert np.count_nonzero(~ok) <= ((order + 1) ** 3 if kind == "inf" else 0) and (kind == "inf") == (not ok.all())
+    if kind == "inf":
+        s["w"][n // 2] = 0.0
+    ref = particles.deposit_rho(s, shape, dx, order)
+    assert field_rel_err([np.where(ok, got, 0.0)], [ref * ok]) < TOL
