@@ -687,6 +687,25 @@ struct EbArgs {
   double scale;
 };
 
+template <class C>
+struct JShiftArgs {
+  CP6<C> in, out;
+  const C* hs[3];
+  int64_t Ny, nzh, nmode;
+};
+// J alone, each component on its own axis: plain DFT -> paper convention, one product per component (in
+// phase_kernel, general, the FP64 form took 0.20 ms for 2.1 million modes)
+template <class C>
+__global__ void __launch_bounds__(256) j_shift_kernel(JShiftArgs<C> a) {
+  const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (m >= a.nmode) return;
+  uint32_t ix, iy, iz;
+  mode_xyz(m, (uint32_t)a.nzh, __ffsll(a.Ny) - 1, ix, iy, iz);
+  const C h[3] = {a.hs[0][ix], a.hs[1][iy], a.hs[2][iz]};
+#pragma unroll
+  for (int c = 0; c < 3; ++c) a.out.p[c][m] = cmul(a.in.p[c][m], h[c]);
+}
+
 template <class C, bool STORE>
 __global__ void __launch_bounds__(256) eb_kernel(EbArgs<C> a) {
   using T = decltype(C().x);
@@ -702,12 +721,16 @@ __global__ void __launch_bounds__(256) eb_kernel(EbArgs<C> a) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) h[c] = cconj(h[c]);
   }
-  h[3] = cmul(h[1], h[2]);
-  h[4] = cmul(h[0], h[2]);
-  h[5] = cmul(h[0], h[1]);
+  // (the scale, a power of two, on the three factors: once per product)
+  const C s1 = STORE ? cscale(h[1], (T)a.scale) : h[1], s2 = STORE ? cscale(h[2], (T)a.scale) : h[2];
+  h[3] = cmul(h[1], s2);
+  h[4] = cmul(h[0], s2);
+  h[5] = cmul(h[0], s1);
+  h[1] = s1;
+  h[2] = s2;
+  if (STORE) h[0] = cscale(h[0], (T)a.scale);
 #pragma unroll
-  for (int c = 0; c < 6; ++c)
-    a.out[c * a.nmode + m] = cmul(a.in[c * a.nmode + m], STORE ? cscale(h[c], (T)a.scale) : h[c]);
+  for (int c = 0; c < 6; ++c) a.out[c * a.nmode + m] = cmul(a.in[c * a.nmode + m], h[c]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1021,6 +1044,18 @@ pic_status psatd_phase_t(pic_ctx* ctx, CP6<C> in, CP6<C> out, const int* comp_ki
   p.nmode = ctx->nmode;
   const int bs = 256;
   dim3 grid((unsigned)((ctx->nmode + bs - 1) / bs), ncomp);
+  if (ncomp == 3 && comp_kind[0] == 6 && comp_kind[1] == 7 && comp_kind[2] == 8 && sign < 0 && scale == 1.0) {
+    JShiftArgs<C> j;
+    j.in = in;
+    j.out = out;
+    for (int a = 0; a < 3; ++a) j.hs[a] = p.hs[a];
+    j.Ny = p.Ny;
+    j.nzh = p.nzh;
+    j.nmode = p.nmode;
+    j_shift_kernel<C><<<grid.x, bs, 0, ctx->stream>>>(j);
+    PIC_LAUNCH_CHECK(ctx);
+    return PIC_OK;
+  }
   phase_kernel<C><<<grid, bs, 0, ctx->stream>>>(p);
   PIC_LAUNCH_CHECK(ctx);
   return PIC_OK;
