@@ -12,8 +12,8 @@
 //   (D f)_{j+1/2} = sum_{n=1}^{m} c_n (f_{j+n} - f_{j-n+1}) / dx,  c_n = alpha^s_{m,n} / (2n - 1),
 // whose Fourier symbol is i [k]_s (Eq. staggered_modified_wave_number); m = 1 is Yee's scheme.
 // curl E is taken at the B positions (E is nodal along the axes it is differentiated along),
-// curl B at the E positions.  One thread per cell; all three components of the updated field
-// in one pass (HBM bound: the neighbours along x and y come from L2).
+// curl B at the E positions.  All three components of the updated field in one pass (the neighbours along
+// x and y come from L2): one thread per cell, or per 16 bytes of z cells where orders and alignment allow it.
 #include "pic_internal.cuh"
 
 #include <cmath>
