@@ -298,7 +298,7 @@ struct UpdArgs {
   int write_j;  // write the Yee-centered J back
 };
 
-// The sums of mode_update in FP64
+// The sums of mode_update in FP64, the field's own term (the largest) last
 template <int VAR>
 __device__ __forceinline__ void fp64_update(const double* k, double c2, const double2 (&cf)[COEF_COUNT], const double2* E,
                                             const double2* B, const double2* J, double2 rn, double2 rp, double2* En,
@@ -325,11 +325,9 @@ __device__ __forceinline__ void fp64_update(const double* k, double c2, const do
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     // B^{n+1} = TC B - i TS [k]xE + i X1 [k]xJ
-    Bn[a] = cfmai(cfmai(cmul(TC, B[a]), cneg(TS), kE[a]), X1, kJ[a]);
+    Bn[a] = cfma(cfmai(cmuli(cmul(X1, kJ[a])), cneg(TS), kE[a]), TC, B[a]);
     // E^{n+1} = TC E + i c^2 TS [k]xB + X4 J + rterm [k]
-    En[a] = cfma(cfmai(cmul(TC, E[a]), c2TS, kB[a]), X4, J[a]);
-    En[a].x = fma(rterm.x, k[a], En[a].x);
-    En[a].y = fma(rterm.y, k[a], En[a].y);
+    En[a] = cfma(cfmai(cfma(cscale(rterm, k[a]), X4, J[a]), c2TS, kB[a]), TC, E[a]);
   }
   if (VAR == 2) {
     const C P1 = cf[COEF_PSI1], P2 = cf[COEF_PSI2], Y1 = cf[COEF_Y1], Y2 = cf[COEF_Y2], Y3 = cf[COEF_Y3],
@@ -339,11 +337,9 @@ __device__ __forceinline__ void fp64_update(const double* k, double c2, const do
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       // <B> = Psi1 B + i Psi2 [k]xE + i Y1 [k]xJ
-      Gb[a] = cfmai(cfmai(cmul(P1, B[a]), P2, kE[a]), Y1, kJ[a]);
+      Gb[a] = cfma(cfmai(cmuli(cmul(Y1, kJ[a])), P2, kE[a]), P1, B[a]);
       // <E> = Psi1 E - i c^2 Psi2 [k]xB + Y4 J + (Y3 rho^n + Y2 rho^{n+1}) [k]
-      Ga[a] = cfma(cfmai(cmul(P1, E[a]), c2P2, kB[a]), Y4, J[a]);
-      Ga[a].x = fma(yr.x, k[a], Ga[a].x);
-      Ga[a].y = fma(yr.y, k[a], Ga[a].y);
+      Ga[a] = cfma(cfmai(cfma(cscale(yr, k[a]), Y4, J[a]), c2P2, kB[a]), P1, E[a]);
     }
   } else {
 #pragma unroll
