@@ -10,6 +10,7 @@
 #include "pic_internal.cuh"
 
 #include <algorithm>
+#include <cfloat>
 
 namespace {
 
@@ -163,9 +164,11 @@ struct Window {
 // a conversion.  The factor 2^-149 is split: w carries 2^-(85 + e), Sz[k] 2^-64 (kFixSz).  A particle
 // whose contributions exceed 2^24 (it holds over 1/64 of its chunk's current) takes e > 0: its
 // contributions are rounded to 2^e, 2^-24 of its largest one, as the FP32 product itself is.  The
-// sign and 2^e go on with one integer multiply by m.  Non-finite amounts deposit 0.  Both factors are
-// >= +0 (move_offset never returns -0, whose pattern would be an integer of its own), and the
-// products are __fmul_rn so that the compiler does not contract them with the weights' formulas.
+// sign and 2^e go on with one integer multiply by m.  Non-finite amounts deposit 0, and particles whose
+// offsets are NaN (moved by a non-finite momentum or field) nothing: their weights' patterns would be
+// integers as well (placed).  Both factors are >= +0 (move_offset never returns -0, whose pattern would be
+// an integer of its own), and the products are __fmul_rn so that the compiler does not contract them with
+// the weights' formulas.
 // Alone (multiply, convert, shared atomic) 15.3 -> 27 lanes per clock per SM; in the push, which its
 // shared-memory wavefronts bound, runs of 10 steps on 128x128x512 cells with 2 per cell went from
 // 29.82 to 29.25 ms and of 6 steps on 256x256x1024 with 1 per cell from 103.1 to 101.0 ms.
@@ -186,6 +189,8 @@ __device__ __forceinline__ Fixed to_fixed(float v, float scale) {
   return f;
 }
 __device__ __forceinline__ int fixed_of(float row, float szs, int m) { return __float_as_int(__fmul_rn(row, szs)) * m; }
+// offsets of move_offset: in [0, 1), or NaN
+__device__ __forceinline__ bool placed(float fx, float fy, float fz) { return fx + fy + fz >= 0.0f; }
 
 // Deposit one particle's (P+1)^3 block: inside the window with shared-memory
 // integer atomics of the contributions rounded to the window's fixed-point scale,
@@ -232,6 +237,7 @@ __device__ __forceinline__ bool deposit_window(const Push32Args& a, const Window
     }
     return false;
   }
+  if (!placed(fx, fy, fz)) return true;
   const int comp = win.comp;
 #pragma unroll
   for (int k = 0; k < NS; ++k) Sz[k] = __fmul_rn(Sz[k], kFixSz);
@@ -313,6 +319,7 @@ __device__ __forceinline__ void deposit_j5(const Push32Args& a, const Window& wi
     }
     return;
   }
+  if (!placed(fx, fy, fz)) return;
   const int comp = win.comp;
   const Fixed f0 = to_fixed<P>(v0, win.sj[0]), f1 = to_fixed<P>(v1, win.sj[1]), f2 = to_fixed<P>(v2, win.sj[2]);
   float Z[NS + 1];  // the block's z weights over the NS + 1 nodes
@@ -772,11 +779,11 @@ __global__ void __launch_bounds__(kTileThreads, 1024 / kTileThreads) push32_tile
     a.ux[p] = ux;
     a.uy[p] = uy;
     a.uz[p] = uz;
+    // (a non-finite amount deposits nothing, and must not take the chunk's scale with it)
     const float qw = fabsf(wp * a.qw_scale);
-    bnd[0] += qw * fabsf(vx);
-    bnd[1] += qw * fabsf(vy);
-    bnd[2] += qw * fabsf(vz);
-    bnd[3] += qw;
+    const float am[4] = {qw * fabsf(vx), qw * fabsf(vy), qw * fabsf(vz), qw};
+#pragma unroll
+    for (int d = 0; d < 4; ++d) bnd[d] += am[d] <= FLT_MAX ? am[d] : 0.0f;
   }
   // Fixed-point scales.  A node sum of component c is at most S_max^3 sum_p |q w v_c| (J) or
   // S_max^3 sum_p |q w| (rho), S_max the largest 1D shape weight; each scale is the power of
