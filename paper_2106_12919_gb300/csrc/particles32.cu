@@ -2035,24 +2035,38 @@ static Key32Args key_args(const pic_ctx* ctx, const pic_species32* sp, const int
   return b;
 }
 
-// scratch of the two-level binning for nsp species: flags, and per species counts (cleared here, and by
-// every binning after use) and cursors
+// Scratch of the two-level binning for nsp species: flags, and per species counts and cursors.  The counts
+// and flags are zero between binnings (every one clears them after use), so a call that failed in
+// between (bin2_dirty) has them cleared here.  Everything a binning needs is allocated before its first
+// launch.
 static pic_status bin32_scratch(pic_ctx* ctx, int nsp) {
-  if (ctx->bin2_species >= nsp) return PIC_OK;
-  // all of them at the first use, as far as they are few: nothing is allocated between two steps
-  const int want = std::max(nsp, std::min(PIC_MAX_BINNED_SPECIES, 2));
-  uint32_t* w = nullptr;
-  const size_t words = 2 * PIC_MAX_BINNED_SPECIES + (size_t)want * 2 * ctx->n_tiles;
-  if (cudaMalloc(&w, words * sizeof(uint32_t)) != cudaSuccess) {
-    cudaGetLastError();
-    return pic_set_error(ctx, PIC_ERR_NOMEM, "binning scratch");
+  const int64_t nt = ctx->n_tiles;
+  const auto words = [nt](int n) { return 2 * PIC_MAX_BINNED_SPECIES + (size_t)n * 2 * nt; };
+  if (nt > kMaxScanTiles && !ctx->cell_counts) {  // the block sums of the scans over several CTAs, and their total
+    const int64_t nblk = (nt + kScanBlock - 1) / kScanBlock;
+    if (cudaMalloc(&ctx->cell_counts, (nblk + 1) * sizeof(uint32_t)) != cudaSuccess) {
+      cudaGetLastError();
+      ctx->cell_counts = nullptr;
+      return pic_set_error(ctx, PIC_ERR_NOMEM, "binning scratch");
+    }
   }
-  if (ctx->bin2) {
-    ctx->bin2_old[ctx->bin2_nold++] = ctx->bin2;  // a captured graph may still use it: freed with the context
+  if (ctx->bin2_species < nsp) {
+    // all of them at the first use, as far as they are few: nothing is allocated between two steps
+    const int want = std::max(nsp, std::min(PIC_MAX_BINNED_SPECIES, 2));
+    uint32_t* w = nullptr;
+    if (cudaMalloc(&w, words(want) * sizeof(uint32_t)) != cudaSuccess) {
+      cudaGetLastError();
+      return pic_set_error(ctx, PIC_ERR_NOMEM, "binning scratch");
+    }
+    if (ctx->bin2) ctx->bin2_old[ctx->bin2_nold++] = ctx->bin2;  // a captured graph may still use it: freed with the context
+    ctx->bin2 = w;
+    ctx->bin2_species = want;
+    ctx->bin2_dirty = 1;
   }
-  ctx->bin2 = w;
-  ctx->bin2_species = want;
-  PIC_CUDA_TRY(ctx, cudaMemsetAsync(w, 0, words * sizeof(uint32_t), ctx->stream));
+  if (ctx->bin2_dirty) {
+    PIC_CUDA_TRY(ctx, cudaMemsetAsync(ctx->bin2, 0, words(ctx->bin2_species) * sizeof(uint32_t), ctx->stream));
+    ctx->bin2_dirty = 0;
+  }
   return PIC_OK;
 }
 
@@ -2096,6 +2110,7 @@ pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_spe
   // grid-stride kernels on a capped grid: when the gate is off they return at once
   const int bs = 256;
   const auto blocks = [&](int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + bs - 1) / bs, 152 * 8)); };
+  ctx->bin2_dirty = 1;  // until the scans, which clear the counts and flags, are enqueued too
   tile_count_kernel<<<dim3(blocks(nmax), (unsigned)n_species), bs, 0, ctx->stream>>>(b);
   PIC_LAUNCH_CHECK(ctx);
   if (nt <= kMaxScanTiles) {
@@ -2104,7 +2119,6 @@ pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_spe
   } else {
     // many small tiles: the scans over several CTAs
     const int64_t nblk = (nt + kScanBlock - 1) / kScanBlock;
-    if (!ctx->cell_counts) PIC_CUDA_TRY(ctx, cudaMalloc(&ctx->cell_counts, (nblk + 2) * sizeof(uint32_t)));
     uint32_t* bsum = ctx->cell_counts;
     uint32_t* total = bsum + nblk;
     for (int q = 0; q < n_species; ++q) {
@@ -2119,6 +2133,7 @@ pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_spe
       PIC_LAUNCH_CHECK(ctx);
     }
   }
+  ctx->bin2_dirty = 0;
   uint32_t* tmp = reinterpret_cast<uint32_t*>(ctx->bin_tmp);
   for (int q = 0; q < n_species; ++q) {
     if (sp[q].n == 0) continue;

@@ -189,6 +189,7 @@ struct pic_ctx {
   // counts and [n_tiles] cursors; outgrown ones are freed with the context
   uint32_t* bin2;
   int bin2_species;
+  int bin2_dirty;  // counts or flags may not be zero (a call failed between their use and their clearing)
   uint32_t* bin2_old[PIC_MAX_BINNED_SPECIES];
   int bin2_nold;
   // tiled FP32 push: nodes its window keeps after the tile along x for the order by cell and the class
