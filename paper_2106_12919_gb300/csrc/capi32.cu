@@ -256,7 +256,8 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
   const bool early_bin = tiled && n_species > 0;
   const int nbin = std::min(n_species, PIC_MAX_BINNED_SPECIES);
   const bool two_level = bin32_two_level(ctx), home = ctx->shape_order == 2 && two_level;
-  const bool linear = tiled && bin32_linear(ctx);
+  bool linear = false;
+  if (tiled) PIC_TRY32(bin32_linear(ctx, &linear));
   if (early_bin) {
     PIC_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
     PIC_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));

@@ -2070,15 +2070,21 @@ static pic_status bin32_scratch(pic_ctx* ctx, int nsp) {
   return PIC_OK;
 }
 
-bool bin32_linear(pic_ctx* ctx) {
-  if (ctx->tile_linear) return ctx->tile_linear == 2;
-  TileArgs t;
-  size_t smem;
-  int n0 = 0, n1 = 0;
-  const bool ok = bin32_two_level(ctx) && choose_layout(ctx, false, t, smem, &n0) == PIC_OK && tile_layout(ctx, t, 2, true) <= (size_t)kMaxTileSmem &&
-         tile_layout(ctx, t, 3, true) <= (size_t)kMaxTileSmem && choose_layout(ctx, true, t, smem, &n1) == PIC_OK && n1 >= n0;
-  ctx->tile_linear = ok ? 2 : 1;
-  return ok;
+pic_status bin32_linear(pic_ctx* ctx, bool* linear) {
+  if (!ctx->tile_linear) {
+    TileArgs t;
+    size_t smem;
+    int n0 = 0, n1 = 0;
+    bool ok = bin32_two_level(ctx) && tile_layout(ctx, t, 3, true) <= (size_t)kMaxTileSmem;
+    if (ok) {
+      PIC_TRY(choose_layout(ctx, false, t, smem, &n0));
+      PIC_TRY(choose_layout(ctx, true, t, smem, &n1));
+      ok = n1 >= n0;
+    }
+    ctx->tile_linear = ok ? 2 : 1;
+  }
+  *linear = ctx->tile_linear == 2;
+  return PIC_OK;
 }
 
 pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_species, int64_t* const* offsets,

@@ -442,7 +442,7 @@ pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_spe
                                 uint32_t* const* chunks, const int* gate, const int* frames, bool home, bool linear);
 // whether the step's binning and push use that order: its shared-memory layout (longer gather rows) must
 // not cost CTAs per SM (8 x 16 x 8 tiles: 3 instead of 4, and they keep the order by cell)
-bool bin32_linear(pic_ctx* ctx);
+pic_status bin32_linear(pic_ctx* ctx, bool* linear);
 // The start of a step of the tiled form, one launch.  advance: after the pushes of the step before,
 // every binned species' tile frame moves by its frame velocity, and the velocity becomes the
 // displacement that at least 3/4 of the species' particles made in that push (else 0).  decide:
