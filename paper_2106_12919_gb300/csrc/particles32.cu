@@ -926,171 +926,11 @@ Push32Args make_args32(pic_ctx* ctx, const pic_species32* sp) {
   return a;
 }
 
-// rho of particles whose neighbours in the array are neighbours in space (sorted ones, or a lattice as
-// laid out), without a binning: a CTA sums the 2048 particles of its chunk in a shared-memory window around
-// them and adds that to rho once, where one thread per particle (push32_kernel) issues (P+1)^3 global
-// atomics, 4 lanes of them per clock per SM at order 3.  Fixed point as in the tiled push; the chunk takes
-// the per-particle global path instead when the window does not fit (an array in random order), and when
-// the sums would be coarser than FP32 ones: the bound of a node's sum is the fullest cell's count times the
-// largest amount times K (the weights a node can have of the cells around it), so the unit is finest where
-// cells and amounts are alike.  Peaks over 16 times the mean load take the global path, as do single
-// particles of less than 1/16 of the chunk's largest amount, non-finite amounts and offsets outside [0, 1).
-// 16.8M particles on 128x128x512, cubic: 0.885 -> 0.470 ms in lattice order, 1.336 -> 0.552 sorted by tile;
-// 68.1M on 256x256x1024: 3.67 -> 2.61 and 6.53 -> 2.17 ms.  Chunks of 4096 with two windows of 115 KB per
-// SM: 0.420 and 0.526, 2.39 and 3.25 ms, but 0.160 instead of 0.125 for 2M on 64x64x256.
-constexpr int kRhoChunk = 2048, kRhoThreads = 512;
-constexpr int kRhoWords = 24 * 1024;  // 96 KB: 2 CTAs per SM
-
-template <int P>
-__global__ void __launch_bounds__(kRhoThreads, 2) rho32_window_kernel(Push32Args a) {
-  extern __shared__ int acc[];
-  __shared__ int s_lo[3], s_hi[3];
-  __shared__ unsigned s_max, s_peak, s_occ, s_n;
-  constexpr int NS = P + 1;
-  const int tid = threadIdx.x;
-  const bool lane0 = (tid & 31) == 0;
-  const int64_t p0 = blockIdx.x * (int64_t)kRhoChunk;
-  const int n = (int)(a.n - p0 < kRhoChunk ? a.n - p0 : kRhoChunk);
-  if (tid < 3) {
-    s_lo[tid] = INT_MAX;
-    s_hi[tid] = INT_MIN;
-  }
-  if (tid == 0) {
-    s_max = s_peak = s_occ = s_n = 0u;
-  }
-  __syncthreads();
-  int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
-  unsigned vmax = 0u;  // bit pattern of the largest |amount|, infinity where the chunk must not be summed here
-  for (int i = tid; i < n; i += kRhoThreads) {
-    const int64_t p = p0 + i;
-    const int c = a.cell[p];
-    const int x[3] = {(c >> (a.shz + a.shy)) & a.mask[0], (c >> a.shz) & a.mask[1], c & a.mask[2]};
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      lo[d] = min(lo[d], x[d]);
-      hi[d] = max(hi[d], x[d]);
-    }
-    const float fx = a.fx[p], fy = a.fy[p], fz = a.fz[p];
-    const bool ok = fx >= 0.f && fx < 1.f && fy >= 0.f && fy < 1.f && fz >= 0.f && fz < 1.f;
-    vmax = max(vmax, ok ? __float_as_uint(a.w[p] * a.qw_scale) & 0x7fffffffu : 0x7f800000u);
-  }
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int l = __reduce_min_sync(0xffffffffu, lo[d]), h = __reduce_max_sync(0xffffffffu, hi[d]);
-    if (lane0) {
-      atomicMin(&s_lo[d], l);
-      atomicMax(&s_hi[d], h);
-    }
-  }
-  vmax = __reduce_max_sync(0xffffffffu, vmax);
-  if (lane0) atomicMax(&s_max, vmax);
-  __syncthreads();
-  // nodes of cells lo..hi: lo - 1 .. hi + 2
-  const int64_t W0 = s_hi[0] - s_lo[0] + 4, W1 = s_hi[1] - s_lo[1] + 4, W2 = s_hi[2] - s_lo[2] + 4;
-  const int ox = s_lo[0] - 1, oy = s_lo[1] - 1, oz = s_lo[2] - 1;
-  const float big = __uint_as_float(s_max);
-  if (s_max == 0u) return;
-  bool window = W0 * W1 * W2 <= kRhoWords && big >= 0x1p-90f && big <= 0x1p100f;
-  const float least = big * 0.0625f;
-  const int w2 = (int)W2, w1 = (int)W1, words = (int)(W0 * W1 * W2);
-  if (window) {
-    for (int i = tid; i < words; i += kRhoThreads) acc[i] = 0;
-    __syncthreads();
-    for (int i = tid; i < n; i += kRhoThreads) {
-      if (!(fabsf(a.w[p0 + i] * a.qw_scale) >= least)) continue;
-      const int c = a.cell[p0 + i];
-      const int x = ((c >> (a.shz + a.shy)) & a.mask[0]) - ox, y = ((c >> a.shz) & a.mask[1]) - oy, z = (c & a.mask[2]) - oz;
-      atomicAdd(acc + (x * w1 + y) * w2 + z, 1);
-    }
-    __syncthreads();
-    unsigned peak = 0u, occ = 0u, sum = 0u;
-    for (int i = tid; i < words; i += kRhoThreads) {
-      const unsigned v = (unsigned)acc[i];
-      peak = max(peak, v);
-      occ += v != 0u;
-      sum += v;
-      acc[i] = 0;
-    }
-    peak = __reduce_max_sync(0xffffffffu, peak);
-    occ = __reduce_add_sync(0xffffffffu, occ);
-    sum = __reduce_add_sync(0xffffffffu, sum);
-    if (lane0) {
-      atomicMax(&s_peak, peak);
-      atomicAdd(&s_occ, occ);
-      atomicAdd(&s_n, sum);
-    }
-    __syncthreads();
-    window = (float)s_peak * (float)s_occ <= 16.0f * (float)s_n;
-  }
-  if (!window) {
-    for (int i = tid; i < n; i += kRhoThreads) {
-      const int64_t p = p0 + i;
-      const int c = a.cell[p];
-      deposit_node_block<P>(a, (c >> (a.shz + a.shy)) & a.mask[0], (c >> a.shz) & a.mask[1], c & a.mask[2], a.fx[p],
-                            a.fy[p], a.fz[p], 0.f, 0.f, 0.f, a.w[p] * a.qw_scale, false);
-    }
-    return;
-  }
-  // power of two with K peak big scale <= 2^30; K: the largest weights of the cells around a node, summed
-  constexpr float K = P == 1 ? 8.01f : (P == 2 ? 5.37f : 4.64f);
-  const float bound = K * (float)s_peak * big;
-  int e;
-  frexpf(bound, &e);
-  e = 30 - e;
-  const float scale = __uint_as_float((uint32_t)(e + 127) << 23);
-  for (int i = tid; i < n; i += kRhoThreads) {
-    const int64_t p = p0 + i;
-    const int c = a.cell[p];
-    const float v = a.w[p] * a.qw_scale;
-    if (!(fabsf(v) >= least)) {
-      deposit_node_block<P>(a, (c >> (a.shz + a.shy)) & a.mask[0], (c >> a.shz) & a.mask[1], c & a.mask[2], a.fx[p],
-                            a.fy[p], a.fz[p], 0.f, 0.f, 0.f, v, false);
-      continue;
-    }
-    int lx, ly, lz;
-    float Sx[NS], Sy[NS], Sz[NS];
-    // (+ 0: an offset of -0 would put the sign bit into a product's pattern)
-    shape32<P>((c >> (a.shz + a.shy)) & a.mask[0], a.fx[p] + 0.0f, lx, Sx);
-    shape32<P>((c >> a.shz) & a.mask[1], a.fy[p] + 0.0f, ly, Sy);
-    shape32<P>(c & a.mask[2], a.fz[p] + 0.0f, lz, Sz);
-    const Fixed f = to_fixed<P>(v, scale);
-    int* const base = acc + ((lx - ox) * w1 + (ly - oy)) * w2 + (lz - oz);
-#pragma unroll
-    for (int k = 0; k < NS; ++k) Sz[k] *= kFixSz;
-#pragma unroll
-    for (int q = 0; q < NS; ++q) {
-#pragma unroll
-      for (int j = 0; j < NS; ++j) {
-        int* const row = base + (q * w1 + j) * w2;
-        const float r = Sx[q] * Sy[j] * f.w;
-#pragma unroll
-        for (int k = 0; k < NS; ++k) atomicAdd(row + k, fixed_of(r, Sz[k], f.m));
-      }
-    }
-  }
-  __syncthreads();
-  const float inv = __uint_as_float((uint32_t)(127 - e) << 23);
-  for (int q = tid >> 5; q < (int)W0 * w1; q += kRhoThreads / 32) {
-    const int x = q / w1, y = q - x * w1;
-    const int64_t row = ((int64_t)((ox + x) & a.mask[0]) * a.Ny + ((oy + y) & a.mask[1])) * a.Nz;
-    for (int z = tid & 31; z < w2; z += 32) {
-      const int v = acc[q * w2 + z];
-      if (v != 0) atomicAdd(a.rho + row + ((oz + z) & a.mask[2]), (float)v * inv);
-    }
-  }
-}
-
-template <int P>
-bool launch_rho32_window(pic_ctx* ctx, const Push32Args& a) {
-  const size_t smem = kRhoWords * sizeof(int);
-  if (cudaFuncSetAttribute(rho32_window_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  rho32_window_kernel<P><<<(unsigned)((a.n + kRhoChunk - 1) / kRhoChunk), kRhoThreads, smem, ctx->stream>>>(a);
-  return true;
-}
-
+// (rho by itself, pic_deposit_rho32, takes push32_kernel too: one thread per particle and an FP32 atomic per
+// node.  Summing it as the tiled push does, in a window of fixed-point sums around each chunk of 2048
+// neighbouring particles, took 0.47 instead of 0.89 ms for 16.8M cubic particles, 1.5% of a 10-step run, but
+// left the nodes beside a chunk's fullest ones with fewer than FP32's 24 bits: errors of 1e-3 to 1 of the
+// node's rho where the density falls off.)
 pic_status launch_push32(pic_ctx* ctx, const Push32Args& a) {
   if (a.n == 0) return PIC_OK;
   const int bs = 256;
@@ -1976,14 +1816,6 @@ pic_status particles_deposit_rho32(pic_ctx* ctx, const pic_species32* sp, float*
   for (int c = 0; c < 3; ++c) a.J[c] = nullptr;
   a.rho = rho;
   a.gather = 0;
-  // below two chunks (the resident CTAs) per SM the windows would leave SMs idle
-  if (a.n >= (int64_t)2 * ctx->nsm * kRhoChunk &&
-      (ctx->shape_order == 1   ? launch_rho32_window<1>(ctx, a)
-       : ctx->shape_order == 2 ? launch_rho32_window<2>(ctx, a)
-                               : launch_rho32_window<3>(ctx, a))) {
-    PIC_LAUNCH_CHECK(ctx);
-    return PIC_OK;
-  }
   return launch_push32(ctx, a);
 }
 
