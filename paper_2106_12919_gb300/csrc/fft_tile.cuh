@@ -105,12 +105,11 @@ __device__ __forceinline__ void dft(C* v) {
   }
 }
 
-// DFT of v_r w_r, w_0 = 1.  FP64, whose transforms are bound by their operations: the second half of the
-// inputs meets the first in multiply-adds, b = p + q w, and the difference is 2 p - b, one per real component:
-// 72 operations instead of 80 at radix 8, 6 instead of 8 at radix 2.  Against long-double transforms of nine
-// grids from 16x8x32 to 8x8x1024 the errors are those of products rounded before the sums, to 1 % either way;
-// radix 4 takes p - q w, which is more exact, where the short form would save 4 of 28.  The field solve on
-// 128x128x256 7.80 -> 7.16 ms, 4 FP64 steps on 64x64x256 10.34 -> 10.13 ms.
+// DFT of v_r w_r, w_0 = 1.  FP64: the second half of the inputs meets the first in multiply-adds, p + q w and p - q w,
+// fewer roundings for the same 80 operations at radix 8 (field solve errors against the exact one 0.5% below
+// those of products rounded before the sums).  The difference as 2 p - (p + q w), one operation per component, would
+// take 72 and the field solve on 128x128x256 7.16 instead of 7.8 ms, but it inherits the sum's rounding: errors 1.3%
+// above.
 template <int R, bool INV, class C>
 __device__ __forceinline__ void dft_twiddled(C* v, const C* __restrict__ t, int stride) {
   const auto tw = [&](int r) {
@@ -126,13 +125,8 @@ __device__ __forceinline__ void dft_twiddled(C* v, const C* __restrict__ t, int 
       const C p = n == 0 ? v[0] : cmul(v[n], tw(n)), q = v[n + H], w = tw(n + H);
       b[n].x = fma(q.x, w.x, fma(-q.y, w.y, p.x));
       b[n].y = fma(q.x, w.y, fma(q.y, w.x, p.y));
-      if (R == 4) {
-        c[n].x = fma(-q.x, w.x, fma(q.y, w.y, p.x));
-        c[n].y = fma(-q.x, w.y, fma(-q.y, w.x, p.y));
-      } else {
-        c[n].x = fma(2.0, p.x, -b[n].x);
-        c[n].y = fma(2.0, p.y, -b[n].y);
-      }
+      c[n].x = fma(-q.x, w.x, fma(q.y, w.y, p.x));
+      c[n].y = fma(-q.x, w.y, fma(-q.y, w.x, p.y));
     }
     if constexpr (R == 8) {
       dft8_rest<INV>(b, c, v);
