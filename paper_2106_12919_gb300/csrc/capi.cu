@@ -148,14 +148,13 @@ void pic_destroy(pic_ctx* ctx) {
                   ctx->rhoh[0], ctx->Jh, ctx->G, ctx->nodal, ctx->Jn, ctx->bin_tid, ctx->bin_counts,
                   ctx->bin_cursor, ctx->bin_tmp, ctx->cell_counts, ctx->cell_cursor, ctx->adj_work, ctx->bin_gate,
                   ctx->bin_outside, ctx->flt1d, ctx->bin_flags, ctx->k1d32, ctx->flt32, ctx->coefq,
-                  ctx->coefq32, ctx->frame, ctx->dhist, ctx->dev_err, ctx->t64_int, ctx->t64_stash, ctx->bin2};
+                  ctx->coefq32, ctx->frame, ctx->dhist, ctx->dev_err, ctx->bin2};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (int q = 0; q < PIC_MAX_BINNED_SPECIES; ++q) {
     if (ctx->sp_off[q]) cudaFree(ctx->sp_off[q]);
     if (ctx->sp_chunk[q]) cudaFree(ctx->sp_chunk[q]);
   }
-  for (int q = 0; q < ctx->t64_nold; ++q) cudaFree(ctx->t64_old[q]);
   for (int q = 0; q < ctx->bin2_nold; ++q) cudaFree(ctx->bin2_old[q]);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
@@ -534,7 +533,7 @@ pic_status pic_step(pic_ctx* ctx, double* const E[3], double* const B[3], double
     PIC_CUDA_TRY(ctx, cudaMemsetAsync(ctx->Jn, 0, 3 * nc * sizeof(double), ctx->stream));
     PIC_CUDA_TRY(ctx, cudaMemsetAsync(rho, 0, nc * sizeof(double), ctx->stream));
     for (int q = 0; q < n_species; ++q) {
-      StageScope t(ctx, STAGE_PUSH, particles_push_launches(ctx, sp[q].n));
+      StageScope t(ctx, STAGE_PUSH, sp[q].n > 0 ? 1 : 0);
       PIC_TRY(particles_push(ctx, En, Bn, &sp[q], Jn, rho));
     }
     CRPtr6 in;

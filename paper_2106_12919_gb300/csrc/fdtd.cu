@@ -314,7 +314,7 @@ pic_status fdtd_step(pic_ctx* ctx, double* const E[3], double* const B[3], doubl
     PIC_CUDA_TRY(ctx, cudaMemsetAsync(ctx->Jn, 0, 3 * nc * sizeof(double), ctx->stream));
     PIC_CUDA_TRY(ctx, cudaMemsetAsync(rho, 0, nc * sizeof(double), ctx->stream));
     for (int q = 0; q < n_species; ++q) {
-      StageScope t(ctx, STAGE_PUSH, particles_push_launches(ctx, sp[q].n));
+      StageScope t(ctx, STAGE_PUSH, sp[q].n > 0 ? 1 : 0);
       PIC_TRY(particles_push(ctx, En, Bn, &sp[q], Jn, rho));
     }
     {

@@ -104,7 +104,6 @@ struct Timers {
   int64_t launches[STAGE_COUNT];
 };
 
-constexpr int kT64Old = 64;
 struct pic_ctx {
   // configuration
   int64_t N[3];
@@ -172,13 +171,6 @@ struct pic_ctx {
   int64_t* bin_counts;   // [n_tiles + 1]
   int64_t* bin_cursor;   // [n_tiles]
   double* bin_tmp;       // [8][bin_cap] permuted copies
-  // tiled FP64 push (grown on demand): particle lists by tile, and [10][t64_cap] deposit positions and
-  // amounts of the particles of the running push
-  int64_t t64_cap;
-  int32_t* t64_int;
-  int64_t* t64_stash;
-  void* t64_old[kT64Old];  // outgrown ones
-  int t64_nold;
   void* scan_tmp;
   size_t scan_tmp_bytes;
   int64_t n_tiles;
@@ -404,7 +396,6 @@ int coef_index(const pic_ctx* ctx, const char* name);
 // particles.cu ----------------------------------------------------------------
 pic_status particles_push(pic_ctx* ctx, const double* const En[3], const double* const Bn[3],
                           const pic_species* sp, double* const J[3], double* rho);
-int particles_push_launches(const pic_ctx* ctx, int64_t n);  // kernel launches of one particles_push call
 pic_status particles_deposit_rho(pic_ctx* ctx, const pic_species* sp, double* rho);
 pic_status particles_bin(pic_ctx* ctx, const pic_species* sp, int64_t* offsets_out);
 pic_status particles_bin_capacity(pic_ctx* ctx, int64_t n);
