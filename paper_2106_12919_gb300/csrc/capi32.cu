@@ -251,11 +251,9 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
   // The first step's (forced) binning reads the particles only: it runs on the
   // context's second stream, concurrently with the entry transforms of the fields on this one,
   // and the first push waits for it (fork / join by events, also valid inside graph capture).
-  // The one-level binning of large tiles leaves a species' sorted copy in scratch that all share, so
-  // there only species 0 is binned early and the others right before their pushes.
   const bool early_bin = tiled && n_species > 0;
   const int nbin = std::min(n_species, PIC_MAX_BINNED_SPECIES);
-  const bool two_level = bin32_two_level(ctx), home = ctx->shape_order == 2 && two_level;
+  const bool home = ctx->shape_order == 2;
   bool linear = false;
   if (tiled) PIC_TRY32(bin32_linear(ctx, &linear));
   if (early_bin) {
@@ -265,11 +263,10 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
     ctx->stream = ctx->aux;
     pic_status st = PIC_OK;
     {
-      StageScope t(ctx, STAGE_BIN, 1 + bin32_launches(ctx, sp, two_level ? nbin : 1));
+      StageScope t(ctx, STAGE_BIN, 1 + bin32_launches(ctx, sp, nbin));
       st = particles_begin32(ctx, sp, n_species, false, true, true, nullptr, nullptr);
       if (st == PIC_OK)
-        st = two_level ? particles_bin32_step(ctx, sp, nbin, ctx->sp_off, ctx->sp_chunk, ctx->bin_gate, ctx->frame, home, linear)
-                       : particles_bin32(ctx, &sp[0], ctx->sp_off[0], ctx->bin_gate, ctx->sp_chunk[0], false, ctx->frame);
+        st = particles_bin32_step(ctx, sp, nbin, ctx->sp_off, ctx->sp_chunk, ctx->bin_gate, ctx->frame, home, linear);
     }
     ctx->stream = main_stream;
     if (st != PIC_OK) return st;
@@ -317,10 +314,10 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
       // also clears J and rho; after the first step the tile frames follow the species' drift (binning
       // stays off while they keep their tiles).  Step 0 is decided (and binned) on the second stream.
       const bool first = s == 0 && early_bin;
-      StageScope t(ctx, STAGE_BIN, 1 + (first || !two_level ? 0 : bin32_launches(ctx, sp, nbin)));
+      StageScope t(ctx, STAGE_BIN, 1 + (first || nbin == 0 ? 0 : bin32_launches(ctx, sp, nbin)));
       PIC_TRY32(particles_begin32(ctx, sp, n_species, s > 0, !first, force, jn, rho));
       if (first) PIC_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
-      else if (two_level && nbin > 0)
+      else if (nbin > 0)
         PIC_TRY32(particles_bin32_step(ctx, sp, nbin, ctx->sp_off, ctx->sp_chunk, ctx->bin_gate, ctx->frame, home, linear));
     } else {
       PIC_CUDA_TRY(ctx, cudaMemsetAsync(jn, 0, 3 * nc * sizeof(float), ctx->stream));
@@ -328,18 +325,10 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
     }
     for (int q = 0; q < n_species; ++q) {
       if (tiled && q < PIC_MAX_BINNED_SPECIES) {
-        // (large tiles) the binning leaves the sorted species in the shared scratch and the push copies
-        // it back, so each species is binned right before its own push
-        if (!two_level && !(s == 0 && q == 0)) {
-          StageScope t(ctx, STAGE_BIN, bin32_launches(ctx, &sp[q], 1));
-          PIC_TRY32(particles_bin32(ctx, &sp[q], ctx->sp_off[q], ctx->bin_gate, ctx->sp_chunk[q], false,
-                                    ctx->frame + 8 * q));
-        }
         // on a grid moving along z two launches: the instantiation for the species' frame velocity
         // works, its twin returns
         StageScope t(ctx, STAGE_PUSH, sp[q].n > 0 ? (ctx->vg[2] != 0.0 ? 2 : 1) : 0);
         PIC_TRY32(particles_push32_tiled(ctx, En, Bn, &sp[q], Jnp, rho, ctx->sp_off[q], ctx->sp_chunk[q],
-                                         two_level ? nullptr : bin32_scatter_gate(ctx),
                                          ctx->frame + 8 * q, ctx->dhist + 10 * q, linear));
       } else {
         StageScope t(ctx, STAGE_PUSH, sp[q].n > 0 ? 1 : 0);

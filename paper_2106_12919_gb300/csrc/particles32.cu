@@ -32,17 +32,8 @@ struct Push32Args {
   float qw_scale;     // q / dV
   int gather;
   int vay;            // 1: Vay's pusher instead of Boris
-  // Tiled push only: when src_gate is set and *src_gate != 0 (the binning ran this step), the
-  // particles are read from the binning's sorted copy src[0..7] (cell, fx, fy, fz, ux, uy, uz, w
-  // as 32-bit words; id_src the ids or null) and written, with w and the ids, to the species
-  // arrays: the push is the copy back of the sort.
-  const int* src_gate;
-  const uint32_t* src[8];
-  const unsigned long long* id_src;
-  unsigned long long* id_dst;
-  float* w_dst;
   // Tiled push only: the species' drift-following tile frame (shift [0..2], velocity [4..6]) and
-  // its displacement counters (see particles_frames_advance); null: no frame
+  // its displacement counters (see particles_begin32); null: no frame
   const int* frame;
   unsigned long long* dhist;
 };
@@ -673,34 +664,12 @@ __global__ void __launch_bounds__(kTileThreads, 1024 / kTileThreads) push32_tile
   // per thread: counts of the cell displacements -1 and +1 per axis in 5-bit fields (a thread
   // visits at most ceil(2048 / 256) + 1 particles of its chunk)
   unsigned dpk = 0u;
-  const bool sorted_src = a.src_gate != nullptr && *a.src_gate != 0;
   for (int j = threadIdx.x; j < q * s; j += blockDim.x) {
     const int pr = interleaved(j, q, s);
     if (pr >= cnt) continue;
     const int p = p0 + pr;
-    int c;
-    float fx, fy, fz, u0x, u0y, u0z, wp;
-    if (sorted_src) {
-      c = (int)a.src[0][p];
-      fx = __uint_as_float(a.src[1][p]);
-      fy = __uint_as_float(a.src[2][p]);
-      fz = __uint_as_float(a.src[3][p]);
-      u0x = __uint_as_float(a.src[4][p]);
-      u0y = __uint_as_float(a.src[5][p]);
-      u0z = __uint_as_float(a.src[6][p]);
-      wp = __uint_as_float(a.src[7][p]);
-      a.w_dst[p] = wp;
-      if (a.id_src) a.id_dst[p] = a.id_src[p];
-    } else {
-      c = a.cell[p];
-      fx = a.fx[p];
-      fy = a.fy[p];
-      fz = a.fz[p];
-      u0x = a.ux[p];
-      u0y = a.uy[p];
-      u0z = a.uz[p];
-      wp = a.w[p];
-    }
+    const int c = a.cell[p];
+    const float fx = a.fx[p], fy = a.fy[p], fz = a.fz[p];
     const int ix = (c >> (a.shz + a.shy)) & a.mask[0], iy = (c >> a.shz) & a.mask[1], iz = c & a.mask[2];
     int lx, ly, lz;
     float Sx[NS], Sy[NS], Sz[NS];
@@ -753,7 +722,7 @@ __global__ void __launch_bounds__(kTileThreads, 1024 / kTileThreads) push32_tile
       }
     }
     float ux, uy, uz;
-    push_u(a, u0x, u0y, u0z, f, ux, uy, uz);
+    push_u(a, a.ux[p], a.uy[p], a.uz[p], f, ux, uy, uz);
     const float ig = rsqrtf(1.0f + (ux * ux + uy * uy + uz * uz) * a.inv_c2);
     const float vx = ux * ig, vy = uy * ig, vz = uz * ig;
     const float dX = a.dtdx[0] * (vx - a.vg[0]), dY = a.dtdx[1] * (vy - a.vg[1]), dZ = a.dtdx[2] * (vz - a.vg[2]);
@@ -780,7 +749,7 @@ __global__ void __launch_bounds__(kTileThreads, 1024 / kTileThreads) push32_tile
     a.uy[p] = uy;
     a.uz[p] = uz;
     // (a non-finite amount deposits nothing, and must not take the chunk's scale with it)
-    const float qw = fabsf(wp * a.qw_scale);
+    const float qw = fabsf(a.w[p] * a.qw_scale);
     const float am[4] = {qw * fabsf(vx), qw * fabsf(vy), qw * fabsf(vz), qw};
 #pragma unroll
     for (int d = 0; d < 4; ++d) bnd[d] += am[d] <= FLT_MAX ? am[d] : 0.0f;
@@ -916,11 +885,6 @@ Push32Args make_args32(pic_ctx* ctx, const pic_species32* sp) {
   a.inv_c2 = (float)(1.0 / (ctx->c * ctx->c));
   a.vay = ctx->pusher == PIC_PUSHER_VAY ? 1 : 0;
   a.qw_scale = (float)(sp->q / (ctx->dx[0] * ctx->dx[1] * ctx->dx[2]));
-  a.src_gate = nullptr;
-  for (int f = 0; f < 8; ++f) a.src[f] = nullptr;
-  a.id_src = nullptr;
-  a.id_dst = nullptr;
-  a.w_dst = nullptr;
   a.frame = nullptr;
   a.dhist = nullptr;
   return a;
@@ -1067,7 +1031,7 @@ pic_status launch_push32_tiled(pic_ctx* ctx, const Push32Args& a, const int64_t*
 // key = tile * cells_per_tile + local cell (z fastest, then x, then y), so particles end up grouped by
 // tile and, inside a tile, ordered by cell (integer only: from the cell index)
 // ---------------------------------------------------------------------------
-// Binning runs only when *gate is non-zero (the device decides, see bin_decide_kernel), so it can
+// The step's binning runs only when *gate is non-zero (the device decides, see begin32_kernel), so it can
 // be enqueued every step without a host round trip.
 __device__ __forceinline__ bool gated_off(const int* gate) { return gate != nullptr && *gate == 0; }
 
@@ -1077,11 +1041,9 @@ __global__ void fill_u32_kernel(uint32_t* p, int64_t n, uint32_t v, const int* g
     p[e] = v;
 }
 
-// scatter gate = binning gate (1 without one) && the keys were out of order: an already sorted
-// species needs its tile ranges but no permutation
-__global__ void scatter_gate_kernel(const int* gate, const int* unsorted, int* sgate) {
-  *sgate = ((gate == nullptr || *gate != 0) && *unsorted != 0) ? 1 : 0;
-}
+// scatter gate = the keys were out of order: an already sorted species needs its tile ranges but no
+// permutation
+__global__ void scatter_gate_kernel(const int* unsorted, int* sgate) { *sgate = *unsorted != 0 ? 1 : 0; }
 
 // What a step of the tiled form does before its binning, in one launch.  Each part is optional.
 //  - advance: after a push, every binned species' tile frame moves by the velocity that push assumed;
@@ -1132,7 +1094,6 @@ __global__ void __launch_bounds__(256) begin32_kernel(Begin32Args a) {
 }
 
 struct Key32Args {
-  const int* gate;
   const int32_t* cell;
   int64_t n;
   int shz, shy;
@@ -1205,7 +1166,6 @@ __device__ __forceinline__ void flag_unsorted(const Key32Args& a, bool mine) {
 }
 
 __global__ void key32_kernel(Key32Args a0) {
-  if (gated_off(a0.gate)) return;
   const Key32Args a = load_frame(a0);
   bool mine = false;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < a.n; p += (int64_t)gridDim.x * blockDim.x)
@@ -1350,8 +1310,7 @@ __device__ __forceinline__ void scatter32_one(const Scatter32Args& a, int64_t p)
   if (a.id_src) a.id_dst[q] = a.id_src[p];
 }
 
-// copy the sorted scratch back into the species arrays (8 words + optional id per particle); used by
-// pic_bin32 only: inside pic_step32 the next tiled push reads the sorted copy instead
+// copy the sorted scratch back into the species arrays (8 words + optional id per particle)
 struct CopyBackArgs {
   const int* gate;
   const uint32_t* src[8];
@@ -1762,13 +1721,6 @@ bool bin32_two_level(const pic_ctx* ctx) {
 constexpr int64_t kMaxScanTiles = 1 << 17;
 
 int bin32_launches(const pic_ctx* ctx, const pic_species32* sp, int n_species) {
-  if (!bin32_two_level(ctx)) {
-    // fill, (keys), three scan kernels, five chunk-list kernels, then the scatter gate, the cursor fill
-    // and the scatter
-    int n = 0;
-    for (int q = 0; q < n_species; ++q) n += 9 + (sp[q].n > 0 ? 4 : 0);
-    return n;
-  }
   int n = 1 + (ctx->n_tiles <= kMaxScanTiles ? 1 : 9 * n_species);
   for (int q = 0; q < n_species; ++q) n += sp[q].n > 0 ? 2 : 0;
   return n;
@@ -1776,7 +1728,7 @@ int bin32_launches(const pic_ctx* ctx, const pic_species32* sp, int n_species) {
 
 bool tiled_push_fits(const pic_ctx* ctx) {
   TileArgs t;
-  return tile_layout(ctx, t, 3, false) <= (size_t)kMaxTileSmem && ctx->ncell < (int64_t(1) << 31);
+  return bin32_two_level(ctx) && tile_layout(ctx, t, 3, false) <= (size_t)kMaxTileSmem && ctx->ncell < (int64_t(1) << 31);
 }
 
 size_t tile_chunk_words(const pic_ctx* ctx, int64_t n) {
@@ -1786,7 +1738,7 @@ size_t tile_chunk_words(const pic_ctx* ctx, int64_t n) {
 
 pic_status particles_push32_tiled(pic_ctx* ctx, const float* const En[3], const float* const Bn[3],
                                   const pic_species32* sp, float* const J[3], float* rho, const int64_t* offsets,
-                                  const uint32_t* chunks, const int* sorted_gate, const int* frame,
+                                  const uint32_t* chunks, const int* frame,
                                   unsigned long long* dhist, bool linear) {
   Push32Args a = make_args32(ctx, sp);
   a.frame = frame;
@@ -1798,15 +1750,6 @@ pic_status particles_push32_tiled(pic_ctx* ctx, const float* const En[3], const 
   }
   a.rho = rho;
   a.gather = 1;
-  if (sorted_gate) {
-    // the binning of this species (if the gate let it run) left its sorted copy in bin_tmp
-    const uint32_t* tmp = reinterpret_cast<const uint32_t*>(ctx->bin_tmp);
-    a.src_gate = sorted_gate;
-    for (int f = 0; f < 8; ++f) a.src[f] = tmp + (int64_t)f * ctx->bin_cap;
-    a.id_src = sp->id ? reinterpret_cast<const unsigned long long*>(ctx->bin_tmp + 4 * ctx->bin_cap) : nullptr;
-    a.id_dst = reinterpret_cast<unsigned long long*>(sp->id);
-    a.w_dst = sp->w;
-  }
   return launch_push32_tiled(ctx, a, offsets, chunks, linear);
 }
 
@@ -1907,7 +1850,7 @@ pic_status bin32_linear(pic_ctx* ctx, bool* linear) {
     TileArgs t;
     size_t smem;
     int n0 = 0, n1 = 0;
-    bool ok = bin32_two_level(ctx) && tile_layout(ctx, t, 3, true) <= (size_t)kMaxTileSmem;
+    bool ok = tile_layout(ctx, t, 3, true) <= (size_t)kMaxTileSmem;
     if (ok) {
       PIC_TRY(choose_layout(ctx, false, t, smem, &n0));
       PIC_TRY(choose_layout(ctx, true, t, smem, &n1));
@@ -2002,12 +1945,11 @@ pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_spe
   return PIC_OK;
 }
 
-pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offsets_out, const int* gate,
-                           uint32_t* chunks_out, bool copy_back, const int* frame) {
+pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offsets_out) {
   const int64_t n = sp->n;
   if (bin32_two_level(ctx)) {
     PIC_TRY(particles_bin_capacity(ctx, 1));  // bin_counts
-    return particles_bin32_step(ctx, sp, 1, &offsets_out, chunks_out ? &chunks_out : nullptr, gate, frame, false, false);
+    return particles_bin32_step(ctx, sp, 1, &offsets_out, nullptr, nullptr, nullptr, false, false);
   }
   PIC_TRY(particles_bin_capacity(ctx, n > 0 ? n : 1));
   const int64_t ncell = ctx->ncell;
@@ -2020,8 +1962,7 @@ pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offse
   uint32_t* bsum = counts + ncell;
   uint32_t* total = bsum + nblk;
   const unsigned fill_blocks = 152 * 8;
-  Key32Args b = key_args(ctx, sp, frame, false);
-  b.gate = gate;
+  Key32Args b = key_args(ctx, sp, nullptr, false);
   b.key = ctx->bin_tid;
   b.counts = counts;
   if (!ctx->bin_flags) PIC_CUDA_TRY(ctx, cudaMalloc(&ctx->bin_flags, 2 * sizeof(int)));
@@ -2029,31 +1970,28 @@ pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offse
   int* sgate = ctx->bin_flags + 1;
   b.unsorted = unsorted;
   PIC_CUDA_TRY(ctx, cudaMemsetAsync(unsorted, 0, sizeof(int), ctx->stream));
-  // grid-stride kernels on a capped grid: when the gate is off they return at once, so a gated
-  // binning costs a few microseconds, not a full-size launch
   const int bs = 256;
   const unsigned nb = (unsigned)std::min<int64_t>((n + bs - 1) / bs, fill_blocks);
   int64_t* tile_off = offsets_out ? offsets_out : ctx->bin_counts;
   // one level: counting sort by cell in tile-major order over the whole grid
-  fill_u32_kernel<<<fill_blocks, 256, 0, ctx->stream>>>(counts, ncell, 0u, gate);
+  fill_u32_kernel<<<fill_blocks, 256, 0, ctx->stream>>>(counts, ncell, 0u, nullptr);
   PIC_LAUNCH_CHECK(ctx);
   if (n > 0) {
     key32_kernel<<<nb, bs, 0, ctx->stream>>>(b);
     PIC_LAUNCH_CHECK(ctx);
   }
-  scan_block_kernel<<<(unsigned)std::min<int64_t>(nblk, 152 * 2), 1024, 0, ctx->stream>>>(counts, ncell, bsum, gate);
+  scan_block_kernel<<<(unsigned)std::min<int64_t>(nblk, 152 * 2), 1024, 0, ctx->stream>>>(counts, ncell, bsum, nullptr);
   PIC_LAUNCH_CHECK(ctx);
-  scan_sums_kernel<<<1, 1024, 0, ctx->stream>>>(bsum, nblk, total, gate);
+  scan_sums_kernel<<<1, 1024, 0, ctx->stream>>>(bsum, nblk, total, nullptr);
   PIC_LAUNCH_CHECK(ctx);
   scan_add_kernel<<<(unsigned)std::min<int64_t>((ncell + 255) / 256, fill_blocks), 256, 0, ctx->stream>>>(
-      counts, ncell, bsum, b.cpt_shift, tile_off, ctx->n_tiles, total, gate);
+      counts, ncell, bsum, b.cpt_shift, tile_off, ctx->n_tiles, total, nullptr);
   PIC_LAUNCH_CHECK(ctx);
-  if (chunks_out) PIC_TRY(build_chunks(ctx, tile_off, chunks_out, gate));
   if (n == 0) {
     PIC_CUDA_TRY(ctx, cudaMemsetAsync(sgate, 0, sizeof(int), ctx->stream));
     return PIC_OK;
   }
-  scatter_gate_kernel<<<1, 1, 0, ctx->stream>>>(gate, unsorted, sgate);
+  scatter_gate_kernel<<<1, 1, 0, ctx->stream>>>(unsorted, sgate);
   PIC_LAUNCH_CHECK(ctx);
   if (!ctx->cell_cursor) PIC_CUDA_TRY(ctx, cudaMalloc(&ctx->cell_cursor, ncell * sizeof(uint32_t)));
   fill_u32_kernel<<<fill_blocks, 256, 0, ctx->stream>>>(ctx->cell_cursor, ncell, 0u, sgate);
@@ -2074,7 +2012,6 @@ pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offse
   s.cursor = ctx->cell_cursor;
   scatter32_kernel<<<nb, bs, 0, ctx->stream>>>(s);
   PIC_LAUNCH_CHECK(ctx);
-  if (!copy_back) return PIC_OK;  // the next tiled push reads the sorted copy
   CopyBackArgs cb;
   cb.gate = sgate;
   for (int f = 0; f < 8; ++f) {

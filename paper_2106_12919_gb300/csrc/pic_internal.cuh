@@ -189,7 +189,7 @@ struct pic_ctx {
   int tile_wx[2];
   int tile_linear;
   int* bin_gate;                    // FP32 form: device flag "re-bin before the next push"
-  int* bin_flags;                   // FP32 binning: [0] keys out of order, [1] scatter gate (see below)
+  int* bin_flags;                   // FP32 binning of large tiles: [0] keys out of order, [1] scatter gate
   unsigned long long* bin_outside;  // FP32 form: particles whose new cell left their tile in the last push
 
   int* dev_err;  // device flag: a bounded wait of a bulk copy gave up (PIC_ERR_TIMEOUT at pic_sync)
@@ -405,30 +405,24 @@ pic_status particles_push32(pic_ctx* ctx, const float* const En[3], const float*
 pic_status particles_deposit_rho32(pic_ctx* ctx, const pic_species32* sp, float* rho);
 // Tiled push: one CTA per chunk of at most kTileChunk particles of one tile, over the ranges
 // offsets[n_tiles + 1] of the last binning; chunks holds the exclusive prefix sum of the
-// tiles' chunk counts [n_tiles + 1], its scan scratch, and the tile of every chunk.  Shared-memory deposit window per chunk.  Correct for any order
-// (out-of-window deposits go global).
+// tiles' chunk counts [n_tiles + 1], its scan scratch, and the tile of every chunk.  Shared-memory deposit window
+// per chunk.  Correct for any order (out-of-window deposits go global).
 constexpr int kTileChunk = 2048;
-bool tiled_push_fits(const pic_ctx* ctx);  // deposit window of the tile fits in shared memory
+// the tile's deposit window fits in shared memory (of no tile above 4096 cells does it: bin32_two_level)
+bool tiled_push_fits(const pic_ctx* ctx);
 size_t tile_chunk_words(const pic_ctx* ctx, int64_t n);  // chunk list size for n particles (words)
 pic_status particles_push32_tiled(pic_ctx* ctx, const float* const En[3], const float* const Bn[3],
                                   const pic_species32* sp, float* const J[3], float* rho, const int64_t* offsets,
-                                  const uint32_t* chunks,
-                                  const int* sorted_gate = nullptr, const int* frame = nullptr,
+                                  const uint32_t* chunks, const int* frame = nullptr,
                                   unsigned long long* dhist = nullptr, bool linear = false);
-// gate: device flag; the binning kernels do nothing while *gate == 0 (nullptr = always bin).
-// chunks_out (optional, tile_chunk_words entries): chunk starts for particles_push32_tiled.
-// copy_back = false leaves the sorted particles in ctx->bin_tmp (the species arrays untouched) for
-// a particles_push32_tiled call with sorted_gate = bin32_scatter_gate(ctx), which reads them there
-// when the binning permuted them and writes the pushed particles to the species arrays.  A species
-// already in key order gets its tile ranges only (no permutation): the scatter gate stays 0.
-// frame (optional): the species' drift-following tile frame (ctx->frame + 8 q); keys are taken from
-// the cell shifted by -frame[0..2].
-pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offsets_out, const int* gate = nullptr,
-                           uint32_t* chunks_out = nullptr, bool copy_back = true, const int* frame = nullptr);
+// pic_bin32.  A species already in key order gets its tile ranges only (no permutation).
+pic_status particles_bin32(pic_ctx* ctx, const pic_species32* sp, int64_t* offsets_out);
 // The same for every species of a step at once (tiles of at most 4096 cells: bin32_two_level); offsets
-// and chunks: one array per species, frames: ctx->frame or nullptr.  home: keys by the nearest node
+// and chunks (for particles_push32_tiled, tile_chunk_words entries): one array per species or nullptr.  gate: device
+// flag; the kernels do nothing while *gate == 0 (nullptr = always bin).  frames: ctx->frame or nullptr (the species'
+// drift-following tile frames: keys are taken from the cell shifted by -frame[0..2]).  home: keys by the nearest node
 // instead of the cell (shape order 2).  linear: the order inside a tile for a push with linear set
-// (class_order_kernel) instead of by cell.  The sorted particles are in the species arrays afterwards.
+// (class_order_kernel), which permutes whatever the order was, instead of by cell.
 pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_species, int64_t* const* offsets,
                                 uint32_t* const* chunks, const int* gate, const int* frames, bool home, bool linear);
 // whether the step's binning and push use that order: its shared-memory layout (longer gather rows) must
@@ -441,13 +435,10 @@ pic_status bin32_linear(pic_ctx* ctx, bool* linear);
 // zero_j, zero_rho (or nullptr): arrays of 3 ncell and ncell floats to clear.
 pic_status particles_begin32(pic_ctx* ctx, const pic_species32* sp, int n_species, bool advance, bool decide, bool force,
                              float* zero_j, float* zero_rho);
-// device flag: the last particles_bin32 call permuted the species (its sorted copy is in bin_tmp)
-inline const int* bin32_scatter_gate(const pic_ctx* ctx) { return ctx->bin_flags + 1; }
 // tiles of at most 4096 cells are binned in two levels (by tile, then by cell inside each tile in
-// shared memory), which always leaves the sorted particles in the species arrays (copy_back is
-// implied); larger tiles by one counting sort over every cell
+// shared memory), larger ones by one counting sort over every cell
 bool bin32_two_level(const pic_ctx* ctx);
-// kernel launches of binning n_species species in a step (for the stage launch counters)
+// kernel launches of particles_bin32_step (for the stage launch counters)
 int bin32_launches(const pic_ctx* ctx, const pic_species32* sp, int n_species);
 
 // center.cu -------------------------------------------------------------------
