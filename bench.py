@@ -437,10 +437,9 @@ def e2e_roundtrip(ctx, fp32, E, B, rho, sp, steps, world, use_graph=True, copy_s
 
 def push_roofline(w, fp32, stage, steps, npart, ncell, clocks, hbm):
     """Roofline of the push stage (gather + Boris + move + deposit: per species and step one push
-    launch in the FP64 form, for shape orders 2 and 3 after three that list the particles by tile; in the
-    FP32 form two, of which the one matching the species' tile-frame velocity works and the other
-    returns at once) against its algorithmic bytes, or for the FP64 form of order 1 its flops, per
-    step."""
+    launch in the FP64 form; in the FP32 form two, of which the one matching the species' tile-frame
+    velocity works and the other returns at once) against its algorithmic bytes (FP32) or flops
+    (FP64) per step."""
     p = w["params"]
     shape = tuple(p["shape"])
     push_ms, push_n = stage["push"]
@@ -468,17 +467,6 @@ def push_roofline(w, fp32, stage, steps, npart, ncell, clocks, hbm):
         return roof
     flops = push_flops_per_particle(p["shape_order"]) * npart
     achieved = flops / push_s_per_step / 1e12
-    if p["shape_order"] >= 2:
-        # the node sums are integer products (no FP64 pipe): 56 B read + 48 B written per particle; nodal E, B
-        # read (48 B) and J, rho deposited (32 B) per cell
-        nbytes = 104 * npart + 80 * ncell
-        return {"kernel": "push64_tile_kernel (gather + Boris + deposit, integer node sums) and its lists by tile, "
-                          "all species' launches of a step",
-                "bound": "hbm", "achieved": nbytes / push_s_per_step / 1e9, "peak": hbm, "unit": "GB/s",
-                "frac": nbytes / push_s_per_step / 1e9 / hbm, "traffic": None,
-                "algorithmic_bytes": "104 B/particle + 80 B/cell per step (%.4g B)" % nbytes,
-                "fp64_equivalent_tflops": achieved,
-                "note": "on chip: issue slots and ALU half busy, shared-memory wavefronts 60%, FP64 pipe 30%"}
     return {"kernel": "push_kernel (gather + Boris + deposit), all species' launches of a step", "bound": "alu",
             "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS,
             "traffic": None, "algorithmic_flops": "22 (p+1)^3 + 250 per particle",
