@@ -90,7 +90,8 @@ __device__ __forceinline__ double wrapd(double x, double L) {
 // The planes of orders 2 and 3 are a rolled loop, their weights in shared memory (wx: per thread Sx, Dx).
 template <int P, bool VAL, class Fn>
 __device__ __forceinline__ void node_grad(const AdjArgs& a, const int* lo, const double (*S)[P + 1],
-                                          const double (*D)[P + 1], const double* wx, double& val, double* grad, Fn&& f) {
+                                          const double (*D)[P + 1], const double* wx, double& val, double* grad,
+                                          Fn&& f) {
   constexpr int NS = P + 1;
   double p0 = 0.0, py0 = 0.0, pz0 = 0.0;  // linear: the first plane's sums
   if (VAL) val = 0.0;

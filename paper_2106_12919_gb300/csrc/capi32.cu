@@ -318,7 +318,8 @@ pic_status pic_step32(pic_ctx* ctx, float* const E[3], float* const B[3], float*
       PIC_TRY32(particles_begin32(ctx, sp, n_species, s > 0, !first, force, jn, rho));
       if (first) PIC_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
       else if (nbin > 0)
-        PIC_TRY32(particles_bin32_step(ctx, sp, nbin, ctx->sp_off, ctx->sp_chunk, ctx->bin_gate, ctx->frame, home, linear));
+        PIC_TRY32(particles_bin32_step(ctx, sp, nbin, ctx->sp_off, ctx->sp_chunk, ctx->bin_gate, ctx->frame, home,
+                                       linear));
     } else {
       PIC_CUDA_TRY(ctx, cudaMemsetAsync(jn, 0, 3 * nc * sizeof(float), ctx->stream));
       PIC_CUDA_TRY(ctx, cudaMemsetAsync(rho, 0, nc * sizeof(float), ctx->stream));

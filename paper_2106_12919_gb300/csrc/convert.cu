@@ -50,7 +50,8 @@ __device__ __forceinline__ int split_cell(double t, float& f) {
   const int i = sh > 52 ? 0 : (int)(m >> (sh & 63));
   const uint64_t r = sh > 52 ? m : m & ((1ull << (sh & 63)) - 1ull);
   const int lz = __clzll((long long)r), ef = 190 - lz - sh;  // the offset's exponent field
-  if (sh < 22 || ef < 1 || r == 0ull) {  // t < 0, t >= 2^31 or not finite (sh < 22, the sign being part of it); tiny or zero offsets
+  // t < 0, t >= 2^31 or not finite (sh < 22, the sign being part of it); tiny or zero offsets
+  if (sh < 22 || ef < 1 || r == 0ull) {
     if (sh >= 22 && r == 0ull) {
       f = 0.0f;
       return i;
@@ -114,7 +115,8 @@ __device__ __forceinline__ double widen(float f) {
 __device__ __forceinline__ double cell_plus(int i, float f) {
   const uint32_t b = __float_as_uint(f), e = b >> 23;
   if ((uint32_t)i >= 1024u || (b != 0u && e - 107u >= 20u)) return (double)i + widen(f);
-  const uint64_t s = ((uint64_t)(uint32_t)i << 52) + (b == 0u ? 0ull : (uint64_t)((b & 0x7fffffu) | 0x800000u) << (e - 98u & 63u));
+  const uint64_t s = ((uint64_t)(uint32_t)i << 52) +
+                     (b == 0u ? 0ull : (uint64_t)((b & 0x7fffffu) | 0x800000u) << (e - 98u & 63u));
   if (s == 0ull) return 0.0;
   const int lz = __clzll((long long)s);
   return __longlong_as_double((int64_t)(((uint64_t)(1034 - lz) << 52) | (s << lz << 1 >> 12)));

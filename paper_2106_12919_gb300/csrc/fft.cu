@@ -36,7 +36,8 @@ using namespace pic_fft;
 __device__ __forceinline__ float halve(float v) { return 0.5f * v; }
 __device__ __forceinline__ double halve(double v) {
   const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff;
-  if ((unsigned)e - 2u > 2044u) return e == 0 && __double2loint(v) == 0 && (hi << 1) == 0 ? v : 0.5 * v;  // 0, subnormal, not finite
+  if ((unsigned)e - 2u > 2044u)  // 0, subnormal, not finite
+    return e == 0 && __double2loint(v) == 0 && (hi << 1) == 0 ? v : 0.5 * v;
   return __hiloint2double(hi - (1 << 20), __double2loint(v));
 }
 

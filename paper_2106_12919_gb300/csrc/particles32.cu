@@ -149,9 +149,9 @@ struct Window {
 // Conversion of a particle's contributions to the window's fixed-point units without a conversion
 // instruction.  float -> int conversions run at 16 lanes per clock per SM (measured; the shared
 // atomics they feed take 30), so 256 of them per cubic particle cost 16 cycles of a pipe that the
-// shared-memory instructions queue with.  Here the product of a weight row and Sz[k] is formed 2^-149 times smaller, so that it is
-// a subnormal float (or one of the first normal binade, which has the same spacing): its bit pattern
-// is the contribution rounded to the nearest integer, exact up to 2^24, and the multiply costs 1/8 of
+// shared-memory instructions queue with.  Here the product of a weight row and Sz[k] is formed 2^-149 times
+// smaller, so that it is a subnormal float (or one of the first normal binade, which has the same spacing):
+// its bit pattern is the contribution rounded to the nearest integer, exact up to 2^24, and the multiply costs 1/8 of
 // a conversion.  The factor 2^-149 is split: w carries 2^-(85 + e), Sz[k] 2^-64 (kFixSz).  A particle
 // whose contributions exceed 2^24 (it holds over 1/64 of its chunk's current) takes e > 0: its
 // contributions are rounded to 2^e, 2^-24 of its largest one, as the FP32 product itself is.  The
@@ -990,7 +990,8 @@ pic_status choose_layout(pic_ctx* ctx, bool linear, TileArgs& t, size_t& smem, i
   return PIC_OK;
 }
 
-pic_status launch_push32_tiled(pic_ctx* ctx, const Push32Args& a, const int64_t* off, const uint32_t* chunk, bool linear) {
+pic_status launch_push32_tiled(pic_ctx* ctx, const Push32Args& a, const int64_t* off, const uint32_t* chunk,
+                               bool linear) {
   if (a.n == 0) return PIC_OK;
   TileArgs t;
   t.off = off;
@@ -1088,7 +1089,8 @@ __global__ void __launch_bounds__(256) begin32_kernel(Begin32Args a) {
     }
   }
   if (a.zero_j)
-    for (int64_t e = t0; e < a.nj / 2; e += nt) reinterpret_cast<float4*>(a.zero_j)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int64_t e = t0; e < a.nj / 2; e += nt)
+      reinterpret_cast<float4*>(a.zero_j)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (a.zero_rho)  // (the caller's array: 8-byte aligned)
     for (int64_t e = t0; e < a.nrho; e += nt) a.zero_rho[e] = make_float2(0.f, 0.f);
 }
@@ -1379,7 +1381,8 @@ struct ClassArgs {
   int plane, row;  // window strides (mod 32)
 };
 __device__ __forceinline__ int class_of(const Key32Args& k, const ClassArgs& c, int key) {
-  const int z = key & k.tmask[2], x = (key >> k.lshift_z) & k.tmask[0], y = (key >> (k.lshift_z + k.lshift_x)) & k.tmask[1];
+  const int z = key & k.tmask[2], x = (key >> k.lshift_z) & k.tmask[0];
+  const int y = (key >> (k.lshift_z + k.lshift_x)) & k.tmask[1];
   return (z + c.plane * x + c.row * y) & 31;
 }
 
@@ -1473,7 +1476,8 @@ __global__ void __launch_bounds__(1024) bin_scan_kernel(BinScan a) {
 }
 
 // after the multi-kernel scan (see particles_bin32): the offsets, scanned in place, become the cursors
-__global__ void scan_finish_kernel(uint32_t* counts, uint32_t* cursor, int64_t n, int* flags, int always, const int* gate) {
+__global__ void scan_finish_kernel(uint32_t* counts, uint32_t* cursor, int64_t n, int* flags, int always,
+                                   const int* gate) {
   if (gated_off(gate)) return;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
     cursor[t] = counts[t];
@@ -1612,8 +1616,8 @@ __global__ void __launch_bounds__(kOrderThreads) cell_order_kernel(TileScatterAr
 // level 2 of the step's binning: scratch -> species arrays, each tile in class order (see ClassArgs).
 // Particle r of class c goes to place sum_c' min(n_c', r) + #{c' < c: n_c' > r}; which particle of a
 // class is its r-th is up to the shared-memory atomics.  Copies as cell_order_kernel.
-__global__ void __launch_bounds__(kOrderThreads) class_order_kernel(TileScatterArgs a, ClassArgs ca, const int64_t* tile_off,
-                                                                    int64_t n_tiles) {
+__global__ void __launch_bounds__(kOrderThreads) class_order_kernel(TileScatterArgs a, ClassArgs ca,
+                                                                    const int64_t* tile_off, int64_t n_tiles) {
   if (gated_off(a.gate) || *a.sgate == 0) return;
   a.k = load_frame(a.k);
   __shared__ uint32_t n[32], next[32];
@@ -1673,8 +1677,8 @@ __global__ void __launch_bounds__(kOrderThreads) class_order_kernel(TileScatterA
 #define PIC_BIN_LIMIT 0.02
 #endif
 
-pic_status particles_begin32(pic_ctx* ctx, const pic_species32* sp, int n_species, bool advance, bool decide, bool force,
-                             float* zero_j, float* zero_rho) {
+pic_status particles_begin32(pic_ctx* ctx, const pic_species32* sp, int n_species, bool advance, bool decide,
+                             bool force, float* zero_j, float* zero_rho) {
   Begin32Args a;
   memset(&a, 0, sizeof(a));
   a.advance = advance ? 1 : 0;
@@ -1728,7 +1732,8 @@ int bin32_launches(const pic_ctx* ctx, const pic_species32* sp, int n_species) {
 
 bool tiled_push_fits(const pic_ctx* ctx) {
   TileArgs t;
-  return bin32_two_level(ctx) && tile_layout(ctx, t, 3, false) <= (size_t)kMaxTileSmem && ctx->ncell < (int64_t(1) << 31);
+  return bin32_two_level(ctx) && tile_layout(ctx, t, 3, false) <= (size_t)kMaxTileSmem &&
+         ctx->ncell < (int64_t(1) << 31);
 }
 
 size_t tile_chunk_words(const pic_ctx* ctx, int64_t n) {
@@ -1833,7 +1838,8 @@ static pic_status bin32_scratch(pic_ctx* ctx, int nsp) {
       cudaGetLastError();
       return pic_set_error(ctx, PIC_ERR_NOMEM, "binning scratch");
     }
-    if (ctx->bin2) ctx->bin2_old[ctx->bin2_nold++] = ctx->bin2;  // a captured graph may still use it: freed with the context
+    // (a captured graph may still use the old one: freed with the context)
+    if (ctx->bin2) ctx->bin2_old[ctx->bin2_nold++] = ctx->bin2;
     ctx->bin2 = w;
     ctx->bin2_species = want;
     ctx->bin2_dirty = 1;
@@ -1890,7 +1896,9 @@ pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_spe
   }
   // grid-stride kernels on a capped grid: when the gate is off they return at once
   const int bs = 256;
-  const auto blocks = [&](int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + bs - 1) / bs, 152 * 8)); };
+  const auto blocks = [&](int64_t n) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + bs - 1) / bs, 152 * 8));
+  };
   ctx->bin2_dirty = 1;  // until the scans, which clear the counts and flags, are enqueued too
   tile_count_kernel<<<dim3(blocks(nmax), (unsigned)n_species), bs, 0, ctx->stream>>>(b);
   PIC_LAUNCH_CHECK(ctx);
@@ -1903,14 +1911,16 @@ pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_spe
     uint32_t* bsum = ctx->cell_counts;
     uint32_t* total = bsum + nblk;
     for (int q = 0; q < n_species; ++q) {
-      scan_block_kernel<<<(unsigned)std::min<int64_t>(nblk, 152 * 2), 1024, 0, ctx->stream>>>(sc.counts[q], nt, bsum, gate);
+      scan_block_kernel<<<(unsigned)std::min<int64_t>(nblk, 152 * 2), 1024, 0, ctx->stream>>>(sc.counts[q], nt, bsum,
+                                                                                              gate);
       PIC_LAUNCH_CHECK(ctx);
       scan_sums_kernel<<<1, 1024, 0, ctx->stream>>>(bsum, nblk, total, gate);
       PIC_LAUNCH_CHECK(ctx);
       scan_add_kernel<<<blocks(nt), 256, 0, ctx->stream>>>(sc.counts[q], nt, bsum, 0, sc.off[q], nt, total, gate);
       PIC_LAUNCH_CHECK(ctx);
       if (chunks) PIC_TRY(build_chunks(ctx, sc.off[q], sc.chunk[q], gate));
-      scan_finish_kernel<<<blocks(nt), 256, 0, ctx->stream>>>(sc.counts[q], sc.cursor[q], nt, flags + 2 * q, sc.always, gate);
+      scan_finish_kernel<<<blocks(nt), 256, 0, ctx->stream>>>(sc.counts[q], sc.cursor[q], nt, flags + 2 * q, sc.always,
+                                                              gate);
       PIC_LAUNCH_CHECK(ctx);
     }
   }
@@ -1936,7 +1946,8 @@ pic_status particles_bin32_step(pic_ctx* ctx, const pic_species32* sp, int n_spe
     if (linear) {
       TileArgs t;
       tile_layout(ctx, t, 3, true);
-      class_order_kernel<<<ob, kOrderThreads, 0, ctx->stream>>>(s, ClassArgs{t.wplane & 31, t.W[2] & 31}, sc.off[q], nt);
+      const ClassArgs c{t.wplane & 31, t.W[2] & 31};
+      class_order_kernel<<<ob, kOrderThreads, 0, ctx->stream>>>(s, c, sc.off[q], nt);
     } else {
       cell_order_kernel<<<ob, kOrderThreads, 0, ctx->stream>>>(s, sc.off[q], nt);
     }

@@ -433,8 +433,8 @@ pic_status bin32_linear(pic_ctx* ctx, bool* linear);
 // displacement that at least 3/4 of the species' particles made in that push (else 0).  decide:
 // *bin_gate = (particles whose new home left their tile in the last tiled push > 2 % of all) || force.
 // zero_j, zero_rho (or nullptr): arrays of 3 ncell and ncell floats to clear.
-pic_status particles_begin32(pic_ctx* ctx, const pic_species32* sp, int n_species, bool advance, bool decide, bool force,
-                             float* zero_j, float* zero_rho);
+pic_status particles_begin32(pic_ctx* ctx, const pic_species32* sp, int n_species, bool advance, bool decide,
+                             bool force, float* zero_j, float* zero_rho);
 // tiles of at most 4096 cells are binned in two levels (by tile, then by cell inside each tile in
 // shared memory), larger ones by one counting sort over every cell
 bool bin32_two_level(const pic_ctx* ctx);

@@ -300,9 +300,9 @@ struct UpdArgs {
 
 // The sums of mode_update in FP64, the field's own term (the largest) last
 template <int VAR>
-__device__ __forceinline__ void fp64_update(const double* k, double c2, const double2 (&cf)[COEF_COUNT], const double2* E,
-                                            const double2* B, const double2* J, double2 rn, double2 rp, double2* En,
-                                            double2* Bn, double2* Ga, double2* Gb) {
+__device__ __forceinline__ void fp64_update(const double* k, double c2, const double2 (&cf)[COEF_COUNT],
+                                            const double2* E, const double2* B, const double2* J, double2 rn,
+                                            double2 rp, double2* En, double2* Bn, double2* Ga, double2* Gb) {
   using C = double2;
   // [k] x F
   const auto cross = [&](const C* F, C* o) {
