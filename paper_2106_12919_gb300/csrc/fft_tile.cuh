@@ -108,7 +108,7 @@ __device__ __forceinline__ void dft(C* v) {
 // DFT of v_r w_r, w_0 = 1.  FP64: the second half of the inputs meets the first in multiply-adds, p + q w and p - q w,
 // fewer roundings for the same 80 operations at radix 8 (field solve errors against the exact one 0.5% below
 // those of products rounded before the sums).  The difference as 2 p - (p + q w), one operation per component, would
-// take 72 and the field solve on 128x128x256 7.16 instead of 7.8 ms, but it inherits the sum's rounding: errors 1.3%
+// take 72 and the field solve on 128x128x256 7.16 instead of 7.54 ms, but it inherits the sum's rounding: errors 1.3%
 // above.
 template <int R, bool INV, class C>
 __device__ __forceinline__ void dft_twiddled(C* v, const C* __restrict__ t, int stride) {
